@@ -60,7 +60,7 @@ __device__ __forceinline__ bool segment_terms(const T *sig_arr, const T *sh_arr,
     const float sig = fmaxf(sraw, 0.f);
     float x[3];
     leaf_sh_dot<K, T>(sh_arr, leaf, Y, x, nullptr);
-    const float e = __expf(-sig * delta);  // same operations as the forward
+    const float e = exp_ftz(-sig * delta);  // same operations as the forward
     const float w = Tr * (1.f - e);
     const float Tn = Tr * e;
     float gs = 0.f;
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kern
                 for (int c = 0; c < 3; ++c) gv.ctot[c] = __ldg(bp.rgb_fwd + 3 * ray + c);
             } else {
                 ShadeVisitor<K, T, false> sv{sig_arr, sh_arr, nullptr, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, nullptr};
-                walk_ray<K, T>(p, sig_arr, sh_arr, stk, ysm, wst, o, d, p.near, p.far, sv);
+                walk_ray<K, T>(p, stk, ysm, wst, o, d, p.near, p.far, sv);
 #pragma unroll
                 for (int c = 0; c < 3; ++c) gv.ctot[c] = fmaf(sv.Tr, p.bg[c], sv.col[c]);
             }
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kern
                 for (int c = 0; c < 3; ++c) gv.g[c] = __ldg(bp.grad_rgb + 3 * ray + c);
             }
             if (gv.g[0] != 0.f || gv.g[1] != 0.f || gv.g[2] != 0.f)
-                walk_ray<K, T>(p, sig_arr, sh_arr, stk, ysm, wst, o, d, p.near, p.far, gv);
+                walk_ray<K, T>(p, stk, ysm, wst, o, d, p.near, p.far, gv);
         }
         if (MODE == kMseTarget) {
 #pragma unroll

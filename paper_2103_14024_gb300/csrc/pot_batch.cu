@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kBlock, POT_RENDER_MIN_BLOCKS) batch_kernel(co
             const T *sig_arr = static_cast<const T *>(it.sigma);
             const T *sh_arr = static_cast<const T *>(it.sh);
             ShadeVisitor<K, T, false> v{sig_arr, sh_arr, nullptr, it.gamma, {0.f, 0.f, 0.f}, 1.f, 0, it.codebook};
-            walk_ray<K, T>(p, sig_arr, sh_arr, stk, ysm, wst, o, d, c->near, c->far, v);
+            walk_ray<K, T>(p, stk, ysm, wst, o, d, c->near, c->far, v);
             const int64_t px = (int64_t)j * it.W + i;
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) it.rgb[3 * px + ch] = fmaf(v.Tr, it.bg[ch], v.col[ch]);

@@ -38,19 +38,29 @@ constexpr int kBrickIndexMinDepth = 3;
 constexpr int kDenseDefaultMaxDepth = 9;  // deeper trees get the brick layout by default
 constexpr int kCellCubeMax = 63;         // largest cube half-extent e the build looks for
 
-// Stored form of an empty entry: the walker's cell shape minus 64 (cube of
-// half-extent e: shape e; node of level l: shape -(1 + D - l)), so that the
-// walker decodes it with one addition; the public form (export) is
-// -(2 + 2 l) / -(3 + 2 e).
-constexpr int kShapeBias = 64;
-__host__ __device__ __forceinline__ int32_t cell_code_node(int level, int D) { return -(1 + D - level) - kShapeBias; }
-__host__ __device__ __forceinline__ int32_t cell_code_cube(int e) { return e - kShapeBias; }
-__host__ __device__ __forceinline__ int cell_code_node_level(int32_t v, int D) { return D + 1 + (v + kShapeBias); }
+// Stored form of an empty entry (negative): what the walker adds to a voxel
+// coordinate to reach the last voxel of the box, as a mask m of low bits to
+// set (an aligned node of m + 1 = 2^(D-l) voxels per axis) and a half-extent e
+// to add (a cube), one of them 0; bit 30 tells a cube from a node.  A leaf
+// entry decodes to m = e = 0.  The public form (export) is -(2 + 2 l) /
+// -(3 + 2 e).
+constexpr int32_t kCellEmpty = (int32_t)0x80000000;
+constexpr int32_t kCellCube = 1 << 30;
+__host__ __device__ __forceinline__ int32_t cell_code_node(int level, int D)
+{
+    return kCellEmpty | ((1 << (D - level)) - 1);
+}
+__host__ __device__ __forceinline__ int32_t cell_code_cube(int e) { return kCellEmpty | kCellCube | (e << 16); }
+__host__ __device__ __forceinline__ int cell_code_node_level(int32_t v, int D)
+{
+    int s = 0;  // of the node's 2^s voxels per axis
+    for (int32_t m = v & 0xFFFF; m; m >>= 1) ++s;
+    return D - s;
+}
 __host__ __device__ __forceinline__ int32_t cell_code_public(int32_t v, int D)
 {
     if (v >= 0) return v;
-    const int s = v + kShapeBias;
-    return s >= 0 ? -(3 + 2 * s) : -(2 + 2 * (D + 1 + s));
+    return v & kCellCube ? -(3 + 2 * ((v >> 16) & 0xFF)) : -(2 + 2 * cell_code_node_level(v, D));
 }
 
 // 4^3 bricks of the grid, ordered x, y, z; inside a brick x, y, z.
@@ -63,10 +73,13 @@ __host__ __device__ __forceinline__ uint32_t in_brick(uint32_t x, uint32_t y, ui
 {
     return ((x & 3u) << 4) | ((y & 3u) << 2) | (z & 3u);
 }
-// Entry of voxel (x, y, z) in the dense layout (D <= 10).
+// Entry of voxel (x, y, z) in the dense layout (D <= 10): brick_of << 6 | in_brick, written with
+// the multiply-adds that leave the walk's busier integer unit free.
 __host__ __device__ __forceinline__ uint32_t cell_index_offset(uint32_t x, uint32_t y, uint32_t z, int D)
 {
-    return (brick_of(x, y, z, D) << 6) | in_brick(x, y, z);
+    const int nb = D > 2 ? D - 2 : 0;
+    return x * 16u + (x >> 2) * ((64u << (2 * nb)) - 64u) + (y * 4u + (y >> 2) * ((64u << nb) - 16u)) +
+           (z + (z >> 2) * 60u);
 }
 __host__ __device__ __forceinline__ int64_t brick_count(int D) { return D > 2 ? 1ll << (3 * (D - 2)) : 1; }
 
@@ -524,22 +537,22 @@ __device__ __forceinline__ void leaf_colour_dot(const T *sh, int64_t leaf, const
     else leaf_sh_dot<K, T>(sh, leaf, Y, x, cb);
 }
 
-// Ask L1 for the lines of one leaf (SH record and sigma) ahead of its use.
-template <int K, typename T>
-__device__ __forceinline__ void prefetch_leaf(const T *sig, const T *sh, int64_t leaf)
+// e^x = 2^(x log2 e) by the base-2 exponential unit, denormals flushed: a
+// transmittance or an exponential below 2^-126 counts as 0 here, and 1 / (1 + e)
+// stays exact to 2 ulp without the range checks that denormals would need.
+__device__ __forceinline__ float exp_ftz(float x)
 {
-    if constexpr (std::is_same<T, cb16>::value) return;
-    else {
-    constexpr int bytes = sh_stride<T>(K) * (int)sizeof(T);
-    const char *r = reinterpret_cast<const char *>(sh + leaf * (int64_t)sh_stride<T>(K));
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(r));
-    if (bytes > 16) asm volatile("prefetch.global.L1 [%0];" ::"l"(r + bytes - 1));
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(sig + leaf));
-    }
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x * 1.44269504089f));
+    return r;
 }
 
-// 1 / (1 + e^-x); x is clamped at -80 (sigmoid < 2e-35) so the divisor stays
-// below 2^126, where the fast division is accurate to 2 ulp.
-__device__ __forceinline__ float sigmoidf_(float x) { return __fdividef(1.f, 1.f + __expf(-fmaxf(x, -80.f))); }
+// 1 / (1 + e^-x); 0 where e^-x overflows.
+__device__ __forceinline__ float sigmoidf_(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + exp_ftz(-x)));
+    return r;
+}
 
 }  // namespace pot

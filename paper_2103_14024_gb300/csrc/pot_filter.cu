@@ -20,7 +20,7 @@ struct MaxWeightVisitor {
     __device__ __forceinline__ bool operator()(int leaf, float delta, const YT &)
     {
         const float sig = fmaxf(Store<T>::load_sigma(sig_arr, leaf), 0.f);
-        const float e = __expf(-sig * delta);
+        const float e = exp_ftz(-sig * delta);
         const float w = Tr * (1.f - e);
         atomicMax(reinterpret_cast<int *>(max_w + leaf), __float_as_int(fmaxf(w, 0.f)));
         Tr *= e;
@@ -34,7 +34,6 @@ __global__ void __launch_bounds__(kBlock, POT_RENDER_MIN_BLOCKS) visibility_kern
     POT_WALK_SHARED(K)
     const int lane = threadIdx.x & 31;
     const T *sig_arr = static_cast<const T *>(p.sigma);
-    const T *sh_arr = static_cast<const T *>(p.sh);
     for (;;) {
         unsigned long long tile = 0;
         if (lane == 0) tile = atomicAdd(p.tile_counter, 1ull);
@@ -44,7 +43,7 @@ __global__ void __launch_bounds__(kBlock, POT_RENDER_MIN_BLOCKS) visibility_kern
         int64_t ray;
         if (tile_ray<true>(p, tile, lane, o, d, near, far, ray)) {
             MaxWeightVisitor<T> v{sig_arr, p.gamma, 1.f, max_w};
-            walk_ray<K, T>(p, sig_arr, sh_arr, stk, ysm, wst, o, d, near, far, v);
+            walk_ray<K, T>(p, stk, ysm, wst, o, d, near, far, v);
         }
     }
 }

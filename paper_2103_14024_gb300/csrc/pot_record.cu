@@ -77,11 +77,11 @@ __global__ void __launch_bounds__(kBlock, POT_RECORD_MIN_BLOCKS)
                 o[r] = __ldg(p.ray_o + 3 * ray + r);
                 d[r] = __ldg(p.ray_d + 3 * ray + r);
             }
-            alive = w.begin(p, stk, sig_arr, sh_arr, o, d, p.near, p.far);
+            alive = w.begin(p, stk, o, d, p.near, p.far);
         }
         while (__any_sync(0xffffffffu, alive)) {
             v.has = false;
-            if (alive) alive = w.step(p, stk, sig_arr, sh_arr, v);
+            if (alive) alive = w.step(p, stk, v);
             const unsigned m = __ballot_sync(0xffffffffu, v.has);
             if (m == 0u || dead) continue;
             const int nseg = __popc(m);
