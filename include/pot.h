@@ -379,8 +379,9 @@ pot_status pot_tree_quantize(const pot_tree *tree, int32_t bits, pot_tree **out,
  * this is its multi-request form).  Each item names its own tree, camera
  * (any resolution), background, early-stop threshold and outputs; items may
  * use different trees, SH degrees and leaf dtypes.  Items are grouped by
- * (SH degree, dtype) and each group is one kernel launch on the stream, whose
- * warps draw 8x4-pixel tiles from all the group's items.  Per-ray arithmetic
+ * (SH degree, dtype, layout of the cell index) and each group is one kernel
+ * launch on the stream, whose warps render the 4x8-pixel tiles of all the
+ * group's items.  Per-ray arithmetic
  * is pot_render's: a request's pixels are identical alone or in a batch.
  * items: host array; rgb [H][W][3] and t_final [H][W] (may be NULL) in device
  * memory; trees on the current device.                                    */

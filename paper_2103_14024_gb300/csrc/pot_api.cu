@@ -39,6 +39,20 @@ unsigned int *device_error_word()
     return ptr[dev];
 }
 
+WalkFrame walk_frame(float size, int depth)
+{
+    int e = 0;
+    std::frexp(size, &e);  // size in [2^(e-1), 2^e)
+    const int k = std::min(1 - e, 126 - kTimeFrac);
+    WalkFrame f;
+    f.ws = std::ldexp(1.f, k);
+    f.size = size * f.ws;
+    f.h = std::ldexp(f.size, -depth);
+    f.invh = 1.f / f.h;
+    f.unit = std::ldexp(1.f, -k - kTimeFrac);
+    return f;
+}
+
 int render_view_group(int n_cams)
 {
     static int g = [] {
@@ -356,8 +370,7 @@ void fill_tree_params(RenderParams &p, const pot_tree *t, const pot_render_opts 
     p.R = 1 << t->desc.depth;
     for (int a = 0; a < 3; ++a) p.lo[a] = t->desc.bbox_lo[a];
     p.size = t->desc.bbox_size;
-    p.h = t->h;
-    p.invh = 1.0f / t->h;
+    p.frame = walk_frame(t->desc.bbox_size, t->desc.depth);
     p.step_cap = 3 * p.R + 16;
     if (o) {
         for (int c = 0; c < 3; ++c) p.bg[c] = o->bg[c];

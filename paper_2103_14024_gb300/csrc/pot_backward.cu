@@ -78,6 +78,7 @@ __device__ __forceinline__ bool segment_terms(const T *sig_arr, const T *sh_arr,
 
 template <int K, typename T>
 struct GradVisitor {
+    static constexpr bool kBasis = true, kVote = false;
     const T *sig_arr;
     const T *sh_arr;
     float gamma;
@@ -167,16 +168,14 @@ struct BackwardParams {
 enum BackwardMode { kGradAndColour = 0, kGrad = 1, kMseTarget = 2 };
 
 #ifndef POT_BACKWARD_MIN_BLOCKS
-// resident blocks per SM: 2 (112 registers); 3 blocks (80 registers, no
-// spills) and 4 (64, small spills) measured slower on 2^18-ray batches of the
-// main tree: 0.96 and 1.39 ms against 0.80 ms for random pixels
-#define POT_BACKWARD_MIN_BLOCKS 2
+// resident blocks per SM: 4 (16 warps, at most 128 registers)
+#define POT_BACKWARD_MIN_BLOCKS 4
 #endif
 
 // MODE kGradAndColour: dL/dC and C given; kGrad: dL/dC given, C from a first
 // walk; kMseTarget: C from a first walk, then dL/dC of the MSE against the
 // target, the loss summed per warp into *loss, C optionally written out.
-template <int K, typename T, int MODE>
+template <int K, typename T, Lookup LOOKUP, int MODE>
 __global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kernel(const BackwardParams bp)
 {
     POT_WALK_SHARED(K)
@@ -192,31 +191,36 @@ __global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kern
         if (tile >= (unsigned long long)p.n_tiles) break;
         const int64_t ray = (int64_t)tile * 32 + lane;
         float lsum = 0.f;  // this ray's squared error (MSE mode)
-        if (ray < p.n_rays) {
-            float o[3], d[3];
+        const bool has = ray < p.n_rays;
+        float o[3], d[3];
+        GradVisitor<K, T> gv;
+        gv.sig_arr = sig_arr;
+        gv.sh_arr = sh_arr;
+        gv.gamma = p.gamma;
+        gv.Tr = 1.f;
+        gv.grad_sigma = bp.grad_sigma;
+        gv.grad_sh = bp.grad_sh;
+        if (has) {
 #pragma unroll
             for (int r = 0; r < 3; ++r) {
                 o[r] = __ldg(p.ray_o + 3 * ray + r);
                 d[r] = __ldg(p.ray_d + 3 * ray + r);
             }
-            GradVisitor<K, T> gv;
-            gv.sig_arr = sig_arr;
-            gv.sh_arr = sh_arr;
-            gv.gamma = p.gamma;
-            gv.Tr = 1.f;
-            gv.grad_sigma = bp.grad_sigma;
-            gv.grad_sh = bp.grad_sh;
+        }
 #pragma unroll
-            for (int c = 0; c < 3; ++c) gv.prefix[c] = 0.f;
-            if (MODE == kGradAndColour) {
+        for (int c = 0; c < 3; ++c) gv.prefix[c] = gv.ctot[c] = gv.g[c] = 0.f;
+        if (MODE == kGradAndColour) {
+            if (has) {
 #pragma unroll
                 for (int c = 0; c < 3; ++c) gv.ctot[c] = __ldg(bp.rgb_fwd + 3 * ray + c);
-            } else {
-                ShadeVisitor<K, T, false> sv{sig_arr, sh_arr, nullptr, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, nullptr};
-                walk_ray<K, T>(p, stk, ysm, wst, o, d, p.near, p.far, sv);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) gv.ctot[c] = fmaf(sv.Tr, p.bg[c], sv.col[c]);
             }
+        } else {
+            ShadeVisitor<K, T, false> sv{sig_arr, sh_arr, nullptr, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, nullptr};
+            walk_rays<K, T, LOOKUP, false>(p, stk, ysm, wst, has, o, d, p.near, p.far, sv);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) gv.ctot[c] = fmaf(sv.Tr, p.bg[c], sv.col[c]);
+        }
+        if (has) {
             if (MODE == kMseTarget) {
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
@@ -229,9 +233,9 @@ __global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kern
 #pragma unroll
                 for (int c = 0; c < 3; ++c) gv.g[c] = __ldg(bp.grad_rgb + 3 * ray + c);
             }
-            if (gv.g[0] != 0.f || gv.g[1] != 0.f || gv.g[2] != 0.f)
-                walk_ray<K, T>(p, stk, ysm, wst, o, d, p.near, p.far, gv);
         }
+        walk_rays<K, T, LOOKUP, false>(p, stk, ysm, wst, has && (gv.g[0] != 0.f || gv.g[1] != 0.f || gv.g[2] != 0.f), o, d, p.near,
+                        p.far, gv);
         if (MODE == kMseTarget) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
@@ -244,18 +248,10 @@ template <typename T>
 cudaError_t launch_backward_t(const BackwardParams &bp, int K, int mode, cudaStream_t s)
 {
     using Fn = void (*)(const BackwardParams);
-    Fn fn = nullptr;
-#define POT_PICK(KK)                                                                              \
-    if (K == KK)                                                                                  \
-        fn = mode == kGradAndColour ? backward_kernel<KK, T, kGradAndColour>                      \
-             : mode == kGrad        ? backward_kernel<KK, T, kGrad>                               \
-                                    : backward_kernel<KK, T, kMseTarget>;
-    POT_PICK(1)
-    POT_PICK(4)
-    POT_PICK(9)
-    POT_PICK(16)
-    POT_PICK(25)
-#undef POT_PICK
+    const bool dense = dense_index(bp.r);
+    Fn fn = mode == kGradAndColour ? POT_PICK_WALK(backward_kernel, K, T, dense, kGradAndColour)
+          : mode == kGrad          ? POT_PICK_WALK(backward_kernel, K, T, dense, kGrad)
+                                   : POT_PICK_WALK(backward_kernel, K, T, dense, kMseTarget);
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = walk_smem_bytes(bp.r.cells == nullptr);
     unsigned grid = 0;
@@ -271,6 +267,8 @@ cudaError_t launch_backward_t(const BackwardParams &bp, int K, int mode, cudaStr
 // delta_i, T_i and P_i, the ray gives dL/dC, C and the SH basis at its
 // direction; GradVisitor then does exactly the per-segment work of the walking
 // backward (same operations, so the same per-segment terms bit for bit).
+
+constexpr int kFlatBlock = 256;  // threads per block of the kernels without a walk
 
 // The per-ray SH basis in registers (the interface of SmemY).
 template <int K>
@@ -328,7 +326,7 @@ __device__ __forceinline__ float run_sum(float v, int lane, int run0)
 // leaf's row gets one set of reductions per warp and step instead of one per
 // record.
 template <int K, typename T>
-__global__ void __launch_bounds__(kBlock, POT_SEGBWD_MIN_BLOCKS) segment_backward_kernel(const SegBackwardParams q)
+__global__ void __launch_bounds__(kFlatBlock, POT_SEGBWD_MIN_BLOCKS) segment_backward_kernel(const SegBackwardParams q)
 {
     if (q.sb.state[1] != 0ull) return;  // the records overflowed: the walking backward runs instead
     const unsigned long long handed = q.sb.state[0];
@@ -423,14 +421,14 @@ cudaError_t launch_segment_backward_t(const SegBackwardParams &q, int K, cudaStr
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kFlatBlock, 0);
     if (e != cudaSuccess) return e;
     // one wave of resident blocks, no more than the slots could need
     int64_t blocks = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
-    const int64_t need = (q.sb.capacity + kBlock - 1) / kBlock;
+    const int64_t need = (q.sb.capacity + kFlatBlock - 1) / kFlatBlock;
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
-    fn<<<(unsigned)blocks, kBlock, 0, s>>>(q);
+    fn<<<(unsigned)blocks, kFlatBlock, 0, s>>>(q);
     count_launch();
     return cudaGetLastError();
 }
@@ -478,7 +476,7 @@ __device__ __forceinline__ int64_t records_used(const SegmentBuffer &sb)
 // that lanes with the same leaf (neighbouring rays of one step) share one
 // atomic, found with a match.
 template <bool SCATTER>
-__global__ void __launch_bounds__(kBlock) leaf_pass_kernel(const SegBinParams q)
+__global__ void __launch_bounds__(kFlatBlock) leaf_pass_kernel(const SegBinParams q)
 {
     if (q.s.sb.state[1] != 0ull) return;
     const int64_t used = records_used(q.s.sb);
@@ -590,15 +588,15 @@ cudaError_t launch_leaf_order_t(const SegBinParams &q, int K, cudaStream_t s)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     // count and scatter passes: a few waves of blocks over the slots (grid-stride)
-    int64_t blocks = (q.s.sb.capacity + kBlock - 1) / kBlock;
+    int64_t blocks = (q.s.sb.capacity + kFlatBlock - 1) / kFlatBlock;
     if (blocks > 8 * (int64_t)sms) blocks = 8 * (int64_t)sms;
     if (blocks < 1) blocks = 1;
     const int64_t n_tiles = (q.n_bins + kScanTile - 1) / kScanTile;
-    leaf_pass_kernel<false><<<(unsigned)blocks, kBlock, 0, s>>>(q);
+    leaf_pass_kernel<false><<<(unsigned)blocks, kFlatBlock, 0, s>>>(q);
     scan_tile_sums_kernel<<<(unsigned)n_tiles, kScanBlock, 0, s>>>(q);
     scan_tile_offsets_kernel<<<1, kScanBlock, 0, s>>>(q, n_tiles);
     scan_apply_kernel<<<(unsigned)n_tiles, kScanBlock, 0, s>>>(q);
-    leaf_pass_kernel<true><<<(unsigned)blocks, kBlock, 0, s>>>(q);
+    leaf_pass_kernel<true><<<(unsigned)blocks, kFlatBlock, 0, s>>>(q);
     count_launch(5);
     // the per-record kernel over the records in leaf order
     SegBackwardParams sq = q.s;
@@ -732,7 +730,7 @@ __global__ void k_step_vec(StepParams sp, float *sigma, float4 *sh4, const float
 // ---- MSE loss of a ray batch: L = mean over n*3 of (rgb - target)^2 --------
 __global__ void k_mse(int64_t n3, const float *rgb, const float *target, float *grad, float *loss)
 {
-    __shared__ float part[kBlock / 32];
+    __shared__ float part[kFlatBlock / 32];
     const float scale = 2.f / (float)n3;
     float acc = 0.f;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n3; j += (int64_t)gridDim.x * blockDim.x) {
@@ -746,7 +744,7 @@ __global__ void k_mse(int64_t n3, const float *rgb, const float *target, float *
     __syncthreads();
     if (threadIdx.x == 0) {
         float s = 0.f;
-        for (int w = 0; w < kBlock / 32; ++w) s += part[w];
+        for (int w = 0; w < kFlatBlock / 32; ++w) s += part[w];
         atomicAdd(loss, s / (float)n3);
     }
 }
@@ -888,7 +886,7 @@ cudaError_t launch_mse(int64_t n, const float *rgb, const float *target, float *
 {
     cudaError_t e = cudaMemsetAsync(loss, 0, sizeof(float), s);
     if (e != cudaSuccess || n == 0) return e;
-    k_mse<<<grid_n(3 * n), kBlock, 0, s>>>(3 * n, rgb, target, grad, loss);
+    k_mse<<<grid_n(3 * n), kFlatBlock, 0, s>>>(3 * n, rgb, target, grad, loss);
     count_launch();
     return cudaGetLastError();
 }

@@ -1,8 +1,8 @@
 // pot_batch.cu -- one launch renders many requests: different trees, cameras,
 // resolutions and outputs (the work list of a continuous-batching server).
 //
-// The host groups the items by (SH coefficients, leaf dtype); each group is one
-// launch.  Every item contributes tiles of kTileW x kTileH pixels (as pot_render);
+// The host groups the items by (SH coefficients, leaf dtype, layout of the cell
+// index); each group is one launch.  Every item contributes tiles of kTileW x kTileH pixels (as pot_render);
 // warps take tiles from one counter and find their item by binary search over
 // the items' first-tile offsets.  The per-ray code (walk + shading) is the
 // same as pot_render's, so a request renders bit-identically alone or in a mix.
@@ -24,10 +24,12 @@ struct BatchItem {
     const void *codebook;
     int depth, R;
     float lo[3];
-    float size, h, invh;
+    float size;
+    WalkFrame frame;
     float bg[3];
     float gamma;
     int W, H, tiles_x;
+    FastDiv by_row;
     int64_t tile_begin;
     float *rgb;
     float *t_final;
@@ -42,8 +44,8 @@ struct BatchParams {
     unsigned int *err;
 };
 
-template <int K, typename T>
-__global__ void __launch_bounds__(kBlock, POT_RENDER_MIN_BLOCKS) batch_kernel(const BatchParams bp)
+template <int K, typename T, Lookup LOOKUP>
+__global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) batch_kernel(const BatchParams bp)
 {
     POT_WALK_SHARED(K)
     const int lane = threadIdx.x & 31;
@@ -69,40 +71,40 @@ __global__ void __launch_bounds__(kBlock, POT_RENDER_MIN_BLOCKS) batch_kernel(co
             hi = min(hi, lo + stride - 1);
         }
         const BatchItem &it = bp.items[lo];
-        const int64_t rem = (int64_t)tile - it.tile_begin;
-        const int ty = (int)(rem / it.tiles_x);
-        const int tx = (int)(rem - (int64_t)ty * it.tiles_x);
+        // 32-bit arithmetic: an item has at most 2^31 pixels
+        const uint32_t rem = (uint32_t)((int64_t)tile - it.tile_begin);
+        const int ty = (int)it.by_row(rem);
+        const int tx = (int)(rem - (uint32_t)ty * (uint32_t)it.tiles_x);
         const int i = tx * kTileW + (lane % kTileW);
         const int j = ty * kTileH + (lane / kTileW);
-        if (i < it.W && j < it.H) {
-            RenderParams p;
-            p.child = it.child;
-            p.cells = it.cells;
-            p.btab = it.btab;
-            p.depth = it.depth;
-            p.R = it.R;
-            p.lo[0] = it.lo[0];
-            p.lo[1] = it.lo[1];
-            p.lo[2] = it.lo[2];
-            p.size = it.size;
-            p.h = it.h;
-            p.invh = it.invh;
-            p.step_cap = 3 * it.R + 16;
-            p.err = bp.err;
-            const pot_camera *c = &it.cam;
-            float o[3], d[3];
-            const float xc = __fdiv_rn(__fsub_rn(__fadd_rn((float)i, 0.5f), c->cx), c->fx);
-            const float yc = -__fdiv_rn(__fsub_rn(__fadd_rn((float)j, 0.5f), c->cy), c->fy);
+        const bool has = i < it.W && j < it.H;
+        RenderParams p;
+        p.child = it.child;
+        p.cells = it.cells;
+        p.btab = it.btab;
+        p.depth = it.depth;
+        p.R = it.R;
+        p.lo[0] = it.lo[0];
+        p.lo[1] = it.lo[1];
+        p.lo[2] = it.lo[2];
+        p.size = it.size;
+        p.frame = it.frame;
+        p.step_cap = 3 * it.R + 16;
+        p.err = bp.err;
+        const pot_camera *c = &it.cam;
+        float o[3], d[3];
+        const float xc = __fdiv_rn(__fsub_rn(__fadd_rn((float)i, 0.5f), c->cx), c->fx);
+        const float yc = -__fdiv_rn(__fsub_rn(__fadd_rn((float)j, 0.5f), c->cy), c->fy);
 #pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                d[r] = __fsub_rn(__fadd_rn(__fmul_rn(c->c2w[r][0], xc), __fmul_rn(c->c2w[r][1], yc)),
-                                 c->c2w[r][2]);
-                o[r] = c->c2w[r][3];
-            }
-            const T *sig_arr = static_cast<const T *>(it.sigma);
-            const T *sh_arr = static_cast<const T *>(it.sh);
-            ShadeVisitor<K, T, false> v{sig_arr, sh_arr, nullptr, it.gamma, {0.f, 0.f, 0.f}, 1.f, 0, it.codebook};
-            walk_ray<K, T>(p, stk, ysm, wst, o, d, c->near, c->far, v);
+        for (int r = 0; r < 3; ++r) {
+            d[r] = __fsub_rn(__fadd_rn(__fmul_rn(c->c2w[r][0], xc), __fmul_rn(c->c2w[r][1], yc)), c->c2w[r][2]);
+            o[r] = c->c2w[r][3];
+        }
+        const T *sig_arr = static_cast<const T *>(it.sigma);
+        const T *sh_arr = static_cast<const T *>(it.sh);
+        ShadeVisitor<K, T, false> v{sig_arr, sh_arr, nullptr, it.gamma, {0.f, 0.f, 0.f}, 1.f, 0, it.codebook};
+        walk_rays<K, T, LOOKUP, true>(p, stk, ysm, wst, has, o, d, c->near, c->far, v);
+        if (has) {
             const int64_t px = (int64_t)j * it.W + i;
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) it.rgb[3 * px + ch] = fmaf(v.Tr, it.bg[ch], v.col[ch]);
@@ -112,11 +114,12 @@ __global__ void __launch_bounds__(kBlock, POT_RENDER_MIN_BLOCKS) batch_kernel(co
 }
 
 template <typename T>
-cudaError_t launch_batch_t(const BatchParams &bp, int K, bool need_stack, cudaStream_t s)
+cudaError_t launch_batch_t(const BatchParams &bp, int K, Lookup look, bool need_stack, cudaStream_t s)
 {
     using Fn = void (*)(const BatchParams);
-    Fn fn = K == 1 ? batch_kernel<1, T> : K == 4 ? batch_kernel<4, T> : K == 9 ? batch_kernel<9, T>
-          : K == 16 ? batch_kernel<16, T> : K == 25 ? batch_kernel<25, T> : nullptr;
+    Fn fn = look == kLookDense ? POT_PICK_K(batch_kernel, K, T, kLookDense)
+          : look == kLookBrick ? POT_PICK_K(batch_kernel, K, T, kLookBrick)
+                               : POT_PICK_K(batch_kernel, K, T, kLookAny);
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = walk_smem_bytes(need_stack);
     const int64_t blocks = (bp.n_tiles + kBlock / 32 - 1) / (kBlock / 32);
@@ -129,13 +132,16 @@ cudaError_t launch_batch_t(const BatchParams &bp, int K, bool need_stack, cudaSt
 
 }  // namespace
 
-// items: host array of n validated requests; groups by (K, dtype), stages the
+// items: host array of n validated requests; groups by (K, dtype, cell index), stages the
 // descriptors and one counter per group in a single stream-ordered buffer.
 cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_t s, unsigned int *err)
 {
     std::vector<int> order(n);
     for (int i = 0; i < n; ++i) order[i] = i;
-    auto key = [&](int i) { return items[i].tree->K * 4 + items[i].tree->desc.leaf_dtype; };
+    auto key = [&](int i) {
+        const pot_tree *t = items[i].tree;
+        return (t->K * 4 + t->desc.leaf_dtype) * 4 + t->cell_kind;
+    };
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return key(a) < key(b); });
     std::vector<BatchItem> desc(n);
     std::vector<int> group_start;
@@ -158,13 +164,13 @@ cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_
         b.R = 1 << t->desc.depth;
         for (int a = 0; a < 3; ++a) b.lo[a] = t->desc.bbox_lo[a];
         b.size = t->desc.bbox_size;
-        b.h = t->h;
-        b.invh = 1.0f / t->h;
+        b.frame = walk_frame(t->desc.bbox_size, t->desc.depth);
         for (int c = 0; c < 3; ++c) b.bg[c] = r.bg[c];
         b.gamma = r.gamma;
         b.W = r.cam.width;
         b.H = r.cam.height;
         b.tiles_x = (b.W + kTileW - 1) / kTileW;
+        b.by_row = fast_div((uint32_t)b.tiles_x);
         b.tile_begin = tiles;
         b.rgb = r.rgb;
         b.t_final = r.t_final;
@@ -194,13 +200,15 @@ cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_
         bp.tile_counter = reinterpret_cast<unsigned long long *>(cb) + g;
         bp.err = err;
         const pot_tree *t = items[order[a]].tree;
-        bool need_stack = false;  // some tree of the group without a cell index
-        for (int k = a; k < b; ++k) need_stack = need_stack || desc[k].cells == nullptr;
+        const Lookup look = t->cell_kind == POT_CELLS_DENSE   ? kLookDense
+                            : t->cell_kind == POT_CELLS_BRICK ? kLookBrick
+                                                              : kLookAny;
+        const bool need_stack = t->cell_kind == POT_CELLS_NONE;
         switch (t->desc.leaf_dtype) {
-        case POT_F32: e = launch_batch_t<float>(bp, t->K, need_stack, s); break;
-        case POT_F16: e = launch_batch_t<__half>(bp, t->K, need_stack, s); break;
-        case POT_CB16: e = launch_batch_t<cb16>(bp, t->K, need_stack, s); break;
-        default: e = launch_batch_t<__nv_bfloat16>(bp, t->K, need_stack, s); break;
+        case POT_F32: e = launch_batch_t<float>(bp, t->K, look, need_stack, s); break;
+        case POT_F16: e = launch_batch_t<__half>(bp, t->K, look, need_stack, s); break;
+        case POT_CB16: e = launch_batch_t<cb16>(bp, t->K, look, need_stack, s); break;
+        default: e = launch_batch_t<__nv_bfloat16>(bp, t->K, look, need_stack, s); break;
         }
     }
     cudaFreeAsync(buf, s);

@@ -121,50 +121,20 @@ __device__ __forceinline__ float df_sub(df a, df b)
 __device__ __forceinline__ bool df_lt(df a, df b) { return __fsub_rn(a.hi, b.hi) < __fsub_rn(b.lo, a.lo); }
 
 // Time t at which o + t d crosses plane k of one axis, i.e.
-// (lo + k h - o) / d, with A = lo - o given exactly as Ahi + Alo and rd = 1/d.
+// (lo + k h - o) / d, with A = lo - o given exactly as Ahi + Alo and rd = 1/d
+// to a few ulp (the remainder is taken exactly and corrected for).  hi and lo
+// stay ordered where the plane's offset from the origin cancels.
 __device__ __forceinline__ df cross_time(int k, float h, float Ahi, float Alo, float d, float rd)
 {
     float p, pe;
     two_prod((float)k, h, p, pe);
-    float s, e;
-    two_sum(Ahi, p, s, e);
-    float rest = __fadd_rn(__fadd_rn(Alo, pe), e);
+    float s0, e;
+    two_sum(Ahi, p, s0, e);
+    const float rest0 = __fadd_rn(__fadd_rn(Alo, pe), e);
+    const float s = __fadd_rn(s0, rest0), rest = __fadd_rn(__fsub_rn(s0, s), rest0);
     float t = __fmul_rn(s, rd);
     float r = __fadd_rn(__fmaf_rn(-t, d, s), rest);
     return {t, __fmul_rn(r, rd)};
-}
-
-// (o + t d) - (lo + k h) on one axis, to ~2^-46 relative: only its sign is used.
-__device__ __forceinline__ float pos_minus_plane(df t, float d, float Ahi, float Alo, int k, float h)
-{
-    float p1, e1;
-    two_prod(t.hi, d, p1, e1);
-    float p2, e2;
-    two_prod((float)k, h, p2, e2);
-    float s, es;
-    two_sum(p1, -Ahi, s, es);
-    float s2, es2;
-    two_sum(s, -p2, s2, es2);
-    float rest = __fsub_rn(__fadd_rn(__fadd_rn(es, es2), __fadd_rn(e1, __fmul_rn(t.lo, d))),
-                           __fadd_rn(Alo, e2));
-    return __fadd_rn(s2, rest);
-}
-
-// Voxel index on one axis of the point o + t d; a point on a face goes to the
-// side the ray is heading (d < 0: lower voxel).  ``margin`` bounds the error of
-// the fp32 estimate in voxel units; only near a face is the exact test run.
-__device__ __forceinline__ int locate_axis(df t, float d, float Ahi, float Alo, float h, float invh,
-                                           float margin)
-{
-    float ug = __fmul_rn(__fmaf_rn(t.hi, d, -Ahi), invh);
-    float kn = rintf(ug);
-    float fr = __fsub_rn(ug, kn);
-    int k = (int)kn;
-    if (fabsf(fr) > margin) return fr > 0.f ? k : k - 1;
-    float v = pos_minus_plane(t, d, Ahi, Alo, k, h);
-    if (v > 0.f) return k;
-    if (v < 0.f) return k - 1;
-    return d < 0.f ? k - 1 : k;
 }
 
 // Exact sign of (p - lo) - k h for fp32 p, lo, h and an integer k (|k| < 2^24):
@@ -547,12 +517,15 @@ __device__ __forceinline__ float exp_ftz(float x)
     return r;
 }
 
-// 1 / (1 + e^-x); 0 where e^-x overflows.
-__device__ __forceinline__ float sigmoidf_(float x)
+// 1 / x to one ulp, denormals flushed.
+__device__ __forceinline__ float rcp_ftz(float x)
 {
     float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + exp_ftz(-x)));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+
+// 1 / (1 + e^-x); 0 where e^-x overflows.
+__device__ __forceinline__ float sigmoidf_(float x) { return rcp_ftz(1.f + exp_ftz(-x)); }
 
 }  // namespace pot

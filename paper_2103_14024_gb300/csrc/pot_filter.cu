@@ -12,6 +12,7 @@ namespace {
 // (non-negative floats order like their bit patterns).
 template <typename T>
 struct MaxWeightVisitor {
+    static constexpr bool kBasis = false, kVote = true;
     const T *sig_arr;
     float gamma;
     float Tr;
@@ -28,8 +29,8 @@ struct MaxWeightVisitor {
     }
 };
 
-template <int K, typename T>
-__global__ void __launch_bounds__(kBlock, POT_RENDER_MIN_BLOCKS) visibility_kernel(const RenderParams p, float *max_w)
+template <int K, typename T, Lookup LOOKUP>
+__global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) visibility_kernel(const RenderParams p, float *max_w)
 {
     POT_WALK_SHARED(K)
     const int lane = threadIdx.x & 31;
@@ -41,10 +42,9 @@ __global__ void __launch_bounds__(kBlock, POT_RENDER_MIN_BLOCKS) visibility_kern
         if (tile >= (unsigned long long)p.n_tiles) break;
         float o[3], d[3], near, far;
         int64_t ray;
-        if (tile_ray<true>(p, tile, lane, o, d, near, far, ray)) {
-            MaxWeightVisitor<T> v{sig_arr, p.gamma, 1.f, max_w};
-            walk_ray<K, T>(p, stk, ysm, wst, o, d, near, far, v);
-        }
+        const bool has = tile_ray<true>(p, tile, lane, o, d, near, far, ray);
+        MaxWeightVisitor<T> v{sig_arr, p.gamma, 1.f, max_w};
+        walk_rays<K, T, LOOKUP, true>(p, stk, ysm, wst, has, o, d, near, far, v);
     }
 }
 
@@ -52,14 +52,15 @@ template <typename T>
 cudaError_t launch_visibility_t(const RenderParams &p, int K, float *max_w, cudaStream_t s)
 {
     using Fn = void (*)(const RenderParams, float *);
-    Fn fn = K == 1 ? visibility_kernel<1, T> : K == 4 ? visibility_kernel<4, T> : K == 9 ? visibility_kernel<9, T>
-          : K == 16 ? visibility_kernel<16, T> : K == 25 ? visibility_kernel<25, T> : nullptr;
+    Fn fn = POT_PICK_WALK(visibility_kernel, K, T, dense_index(p));
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = walk_smem_bytes(p.cells == nullptr);
     unsigned grid = 0;
     cudaError_t e = persistent_grid(fn, smem, p.n_tiles, 0, &grid);
     if (e != cudaSuccess) return e;
-    fn<<<grid, kBlock, smem, s>>>(p, max_w);
+    RenderParams q = p;
+    set_tile_divs(q);
+    fn<<<grid, kBlock, smem, s>>>(q, max_w);
     count_launch();
     return cudaGetLastError();
 }

@@ -39,6 +39,40 @@ namespace pot {
 constexpr int kTileW = POT_TILE_W;
 constexpr int kTileH = 32 / POT_TILE_W;
 
+// n / d for 32-bit n and a divisor fixed before the launch: a high product and
+// two shifts (Granlund and Montgomery, "Division by invariant integers using
+// multiplication", PLDI 1994, figure 4.1) instead of a division per thread.
+struct FastDiv {
+    uint32_t mul, sh1, sh2;
+    __host__ __device__ uint32_t operator()(uint32_t n) const
+    {
+#ifdef __CUDA_ARCH__
+        const uint32_t t = __umulhi(mul, n);
+#else
+        const uint32_t t = (uint32_t)(((uint64_t)mul * n) >> 32);
+#endif
+        return (t + ((n - t) >> sh1)) >> sh2;
+    }
+};
+inline FastDiv fast_div(uint32_t d)
+{
+    int l = 0;  // ceil(log2 d)
+    while (l < 32 && (1ull << l) < d) ++l;
+    return {(uint32_t)(((1ull << 32) * ((1ull << l) - d)) / d + 1), (uint32_t)(l < 1 ? l : 1), (uint32_t)(l > 0 ? l - 1 : 0)};
+}
+
+// The tree's box in the scale of the walk: lengths times the power of two ws
+// that brings the box's edge into [1, 2) (exact products, whatever the box's
+// size; capped where a time unit's length would fall below the normal floats).
+struct WalkFrame {
+    float ws;       // scale
+    float size, h;  // edges of the box and of a voxel, scaled
+    float invh;     // 1 / h, scaled
+    float unit;     // world length of 2^-kTimeFrac scaled lengths
+};
+constexpr int kTimeFrac = 49;
+WalkFrame walk_frame(float size, int depth);
+
 // Everything a render launch needs; passed by value.
 struct RenderParams {
     const int32_t *child;
@@ -51,8 +85,7 @@ struct RenderParams {
     int R;
     float lo[3];
     float size;
-    float h;
-    float invh;
+    WalkFrame frame;
     float bg[3];
     float gamma;
     int step_cap;
@@ -63,6 +96,7 @@ struct RenderParams {
     int W, H;
     int tiles_x;
     int64_t tiles_per_cam;
+    FastDiv by_group, by_view, by_last, by_row;  // tiles per view group, views per group and in the last one, tiles_x
     const float *ray_o;
     const float *ray_d;
     int64_t n_rays;
@@ -77,6 +111,16 @@ struct RenderParams {
     unsigned long long *tile_counter;
     unsigned int *err;
 };
+
+// The divisors of tile numbers, from the camera fields (view_group, n_cams, tiles).
+inline void set_tile_divs(RenderParams &p)
+{
+    const int last = p.n_cams % p.view_group;
+    p.by_group = fast_div((uint32_t)(p.tiles_per_cam * p.view_group));
+    p.by_view = fast_div((uint32_t)p.view_group);
+    p.by_last = fast_div((uint32_t)(last ? last : p.view_group));
+    p.by_row = fast_div((uint32_t)p.tiles_x);
+}
 
 // Launches (defined in pot_render_*.cu); return the CUDA error of the launch.
 cudaError_t launch_render_f32(const RenderParams &p, int K, bool cams, bool count, cudaStream_t s,

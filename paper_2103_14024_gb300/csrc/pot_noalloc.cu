@@ -174,8 +174,7 @@ pot_status pot_render_noalloc(const pot_tree *t, const pot_camera *cams, int32_t
     p.R = 1 << t->desc.depth;
     for (int a = 0; a < 3; ++a) p.lo[a] = t->desc.bbox_lo[a];
     p.size = t->desc.bbox_size;
-    p.h = t->h;
-    p.invh = 1.0f / t->h;
+    p.frame = walk_frame(t->desc.bbox_size, t->desc.depth);
     p.step_cap = 3 * p.R + 16;
     if (opts) {
         for (int c = 0; c < 3; ++c) p.bg[c] = opts->bg[c];

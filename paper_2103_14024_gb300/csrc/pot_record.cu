@@ -14,7 +14,7 @@
 #include "pot_segments_internal.h"
 
 #ifndef POT_RECORD_MIN_BLOCKS
-#define POT_RECORD_MIN_BLOCKS 3  // resident blocks per SM: 80 registers, no spills (64 registers spill 28 bytes)
+#define POT_RECORD_MIN_BLOCKS 6  // resident blocks per SM: 80 registers, no spills
 #endif
 
 namespace pot {
@@ -42,7 +42,7 @@ struct RecordVisitor {
     }
 };
 
-template <int K, typename T>
+template <int K, typename T, Lookup LOOKUP>
 __global__ void __launch_bounds__(kBlock, POT_RECORD_MIN_BLOCKS)
     record_kernel(const RenderParams p, const SegmentBuffer sb)
 {
@@ -66,19 +66,21 @@ __global__ void __launch_bounds__(kBlock, POT_RECORD_MIN_BLOCKS)
         RecordVisitor<K, T> v;
         v.sv = ShadeVisitor<K, T, false>{sig_arr, sh_arr, nullptr, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, nullptr};
         v.has = false;
-        Walker<K, T> w;
+        Walker<K, T, LOOKUP> w;
         w.ysm = ysm;
         w.st = wst;
-        bool alive = false;
-        if (ray < p.n_rays) {
-            float o[3], d[3];
+        bool alive = ray < p.n_rays;
+        float o[3], d[3];
+        if (alive) {
 #pragma unroll
             for (int r = 0; r < 3; ++r) {
                 o[r] = __ldg(p.ray_o + 3 * ray + r);
                 d[r] = __ldg(p.ray_d + 3 * ray + r);
             }
-            alive = w.begin(p, stk, o, d, p.near, p.far);
         }
+        float u[3] = {0.f, 0.f, 1.f};
+        alive = alive && w.begin(p, stk, o, d, p.near, p.far, u);
+        if (alive) w.basis(u);
         while (__any_sync(0xffffffffu, alive)) {
             v.has = false;
             if (alive) alive = w.step(p, stk, v);
@@ -126,8 +128,7 @@ template <typename T>
 cudaError_t launch_record_t(const RenderParams &p, const SegmentBuffer &sb, int K, cudaStream_t s)
 {
     using Fn = void (*)(const RenderParams, const SegmentBuffer);
-    Fn fn = K == 1 ? record_kernel<1, T> : K == 4 ? record_kernel<4, T> : K == 9 ? record_kernel<9, T>
-          : K == 16 ? record_kernel<16, T> : K == 25 ? record_kernel<25, T> : nullptr;
+    Fn fn = POT_PICK_WALK(record_kernel, K, T, dense_index(p));
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = walk_smem_bytes(p.cells == nullptr);
     unsigned grid = 0;

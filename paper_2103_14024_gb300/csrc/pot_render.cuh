@@ -25,41 +25,56 @@
 
 namespace pot {
 
-constexpr int kBlock = 256;
+// How a walk finds the cell of a voxel: the dense cell index, its brick
+// layout, or whichever the tree has (the descent of the child array included).
+enum Lookup { kLookDense, kLookBrick, kLookAny };
+
+// Threads per block of the walk kernels, and the blocks per SM that their
+// register budget is cut for: 6 blocks, 24 warps, 80 registers with the dense
+// index.  The walk and the shading need about 75; at 64 registers (32 warps) the
+// loop spills, which lone views, bound by the latency of their longest rays,
+// pay for (256 x 256 f16 109 against 89 us, 800 x 800 f32 350 against 320 us)
+// and full launches do not notice (40 views: f16 5.68 against 5.65 ms, f32 7.31
+// against 7.32 ms).  72 registers (28 warps): 89 us, 340 us, 5.65 ms, 7.33 ms.
+// With bricks a step waits for two loads in turn, and 32 warps are better (one
+// full-HD view at depth 10: 768 against 801 us).
+constexpr int kBlock = 128;
 #ifndef POT_RENDER_MIN_BLOCKS
-#define POT_RENDER_MIN_BLOCKS 4  // resident blocks per SM the register budget is cut for (64 registers)
+#define POT_RENDER_MIN_BLOCKS 6
 #endif
+constexpr int render_min_blocks(Lookup l) { return l == kLookDense ? POT_RENDER_MIN_BLOCKS : 8; }
 
 // Fixed-point ray times.  A walk measures time from the clip range's entry
-// tin in units of 2^-s, s such that the whole clip range [tin, tout] is at
-// least 2^49 and below 2^50 units, and keeps it in 64-bit integers.  The
+// tin in units of 2^-kTimeFrac, with the ray's direction scaled by a power of
+// two to a length in [1, 2) and the box to an edge in [1, 2) (WalkFrame), and
+// keeps it in 64-bit integers: the clip range is below 2^51 units.  The
 // crossing times of one axis's planes are then an arithmetic progression
 // nx, nx + hs, nx + 2 hs, ... whose terms are exact sums: advancing by one
 // plane, or by the j planes of a box, gives the same time whichever way the
 // plane is reached, so leaf segments do not depend on how empty space is
 // stepped over, and comparisons need no error bounds.  nx and hs are rounded
-// from double-float values once per ray (a voxel is about 2^41 units at
-// depth 9 and 2^38 at depth 12: rounding hs moves a crossing by at most 2^-33
-// and 2^-27 of a voxel, the double-float inputs by about as much).
+// from double-float values once per ray (a voxel is at least 2^39 units at
+// depth 9 and 2^36 at depth 12: rounding hs moves a crossing by at most 2^-31
+// and 2^-25 of a voxel).
 // Axes along which the ray does not move, and planes it would reach only after
-// its range, have nx or hs = kTimeNever; nx + j hs stays below 2^63 for every
-// j < 2^kMaxDepth.
-constexpr int64_t kTimeNever = 1ll << 50;
-constexpr int kTimeRangeExp = 49;
+// its range, have nx or hs = kTimeNever; nx + j hs stays below 2^63 for the
+// j < 2^11 planes of any box.
+constexpr int64_t kTimeNever = 1ll << 51;
+constexpr float kTimeScale = (float)(1ll << kTimeFrac);
 
-// (a - tin) 2^s, not below 0, s split into the factors s1 s2 so that neither
-// overflows.  (The parts of a crossing time need not be ordered: where a
-// plane's offset from the origin cancels, all of it is in a.lo.)
-__device__ __forceinline__ int64_t fixed_time(df a, df tin, float s1, float s2)
+// hi + lo (lo below hi's last bits, or both small) in time units.
+__device__ __forceinline__ int64_t fixed_time(float hi, float lo)
 {
-    float ah, al, hi, e;
-    two_sum(a.hi, a.lo, ah, al);
-    two_sum(ah, -tin.hi, hi, e);
-    const float lo = __fadd_rn(e, __fsub_rn(al, tin.lo));
-    const float f = __fmul_rn(__fmul_rn(hi, s1), s2);
+    const float f = __fmul_rn(hi, kTimeScale);
     if (!(f < (float)kTimeNever)) return kTimeNever;  // also NaN
-    const int64_t t = __float2ll_rn(fmaxf(f, -(float)kTimeNever)) + __float2ll_rn(__fmul_rn(__fmul_rn(lo, s1), s2));
-    return t < 0 ? 0 : t;
+    if (f < -(float)kTimeNever) return -kTimeNever;
+    return __float2ll_rn(f) + __float2ll_rn(__fmul_rn(lo, kTimeScale));
+}
+__device__ __forceinline__ int64_t fixed_time_since(df a, df tin)
+{
+    float hi, e;
+    two_sum(a.hi, -tin.hi, hi, e);
+    return fixed_time(hi, __fadd_rn(e, __fsub_rn(a.lo, tin.lo)));
 }
 
 __device__ __forceinline__ float exp2_int(int x) { return __int_as_float((127 + x) << 23); }
@@ -90,17 +105,24 @@ __device__ __forceinline__ float exp2_int(int x) { return __int_as_float((127 + 
 // for empty boxes and leaves (lanes at a leaf wait for the others: 8.32 ms for
 // f16), one shared exit-time computation for both kinds of cell (6.28 against
 // 6.05 ms).
-template <int K, typename T>
+//
+// LOOKUP: how cells are found, fixed for the kernels where it pays (kLookAny
+// asks the tree).  It saves branches, but matters more for the load of the next
+// entry: where several lookups meet, the loaded register is copied, and the
+// copy waits for the load before the shading's loads are issued (40 views, f16:
+// 6.05 -> 5.68 ms; one full-HD view of a depth-10 tree with bricks: 807 -> 768 us).
+template <int K, typename T, Lookup LOOKUP>
 struct Walker {
+    static constexpr bool DENSE = LOOKUP == kLookDense, BRICK = LOOKUP == kLookBrick;
     int64_t nx[3], hs[3];  // time of the next plane and between planes, per axis
     int64_t t, tout;
     int q[3];              // mirrored voxel
     uint32_t flip;         // the mirror, in the form of the tree's cell lookup
     float unit;            // world length of one time unit
     int cell;              // entry of voxel q: leaf >= 0, or an empty box (cell_code_*)
-    int lvl_valid, step_i;
+    int step_i;
     // rows of shared memory: the per-ray SH basis, and 1 / hs per axis (read
-    // only where a box of more than one voxel is left), which saves registers
+    // only where an empty box is left), which saves registers
     float *ysm;
     float4 *st;
     __device__ __forceinline__ SmemY<K, kBlock> Y() const { return {ysm}; }
@@ -108,12 +130,12 @@ struct Walker {
     // a3: the entry of mirrored voxel q: one load from the cell index when the
     // tree has one (two in the brick layout), else a descent from the deepest
     // ancestor q shares with voxel pq (whose path the stack holds up to
-    // lvl_valid)
+    // the level in its last row)
     __device__ __forceinline__ int locate(const RenderParams &p, int32_t *stk, const int pq[3])
     {
         const int D = p.depth;
-        if (p.cells) {
-            if (!p.btab)
+        if (DENSE || BRICK || p.cells) {
+            if (DENSE || (!BRICK && !p.btab))
                 return __ldg(p.cells + (cell_index_offset((uint32_t)q[0], (uint32_t)q[1], (uint32_t)q[2], D) ^ flip));
             const uint32_t bk = brick_of((uint32_t)q[0], (uint32_t)q[1], (uint32_t)q[2], D);
             const uint32_t in = in_brick((uint32_t)q[0], (uint32_t)q[1], (uint32_t)q[2]);
@@ -124,7 +146,7 @@ struct Walker {
         }
         const unsigned diff = (unsigned)((q[0] ^ pq[0]) | (q[1] ^ pq[1]) | (q[2] ^ pq[2]));
         const int lc = diff ? D - 32 + __clz(diff) : D - 1;  // level of the common ancestor
-        int l = min(lc, lvl_valid);
+        int l = min(lc, stk[kMaxDepth * kBlock]);
         int node = stk[l * kBlock];
         int out = 0;
         for (; l < D; ++l) {
@@ -139,89 +161,152 @@ struct Walker {
             out = c < 0 ? -c - 1 : cell_code_node(l + 1, D);  // an empty slot: an empty node of level l + 1
             break;
         }
-        lvl_valid = min(l, D - 1);
+        stk[kMaxDepth * kBlock] = min(l, D - 1);
         return out;
     }
 
-    __device__ __forceinline__ bool begin(const RenderParams &p, int32_t *stk, const float o[3], const float d[3],
-                                          float near, float far)
+    // Leaves the unit direction in the first three floats of the basis row.
+    __device__ __forceinline__ bool begin(const RenderParams &p, int32_t *stk, const float o[3], const float dw[3],
+                                          float near, float far, float u[3])
     {
         const int R = p.R;
-        const float h = p.h, invh = p.invh;
-        const float len = sqrtf(fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2])));
+        const float h = p.frame.h, invh = p.frame.invh;
+        const float len = sqrtf(fmaf(dw[0], dw[0], fmaf(dw[1], dw[1], dw[2] * dw[2])));
         if (!(len > 0.f) || !(len < 3.0e38f)) return false;
         const float invlen = __frcp_rn(len);
-        {
-            float Yt[K];
-            sh_basis<K>(d[0] * invlen, d[1] * invlen, d[2] * invlen, Yt);
-            SmemY<K, kBlock>::store(ysm, Yt);
-        }
-        float Ahi[3], Alo[3], rd[3];  // A = lo - o exactly, 1 / d
+#pragma unroll
+        for (int a = 0; a < 3; ++a) u[a] = dw[a] * invlen;
+        // the direction scaled to a length in [1, 2)
+        const int el = (int)(__float_as_uint(len) >> 23) - 127;
+        const float ds = exp2_int(-el), il = invlen * exp2_int(el);
+        unit = __fmul_rn(__fmul_rn(len, ds), p.frame.unit);
+        float d[3], rd[3], Ahi[3], Alo[3], th[3], tl[3];  // A = lo - o exactly, 1 / d, time across the box
+        bool move[3];
+        // a2: clip range in scaled time (position o + t d)
+        df tin = {near * p.frame.ws * il, 0.f}, tend = {far * p.frame.ws * il, 0.f};
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             two_sum(p.lo[a], -o[a], Ahi[a], Alo[a]);
-            rd[a] = d[a] != 0.f ? __frcp_rn(d[a]) : 0.f;
-        }
-        // a2: clip range in units of the ray parameter t (position o + t d)
-        df tin = {near * invlen, 0.f}, tend = {far * invlen, 0.f};
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (d[a] == 0.f) {
-                float s, e;
-                two_sum(o[a], -p.lo[a], s, e);
+            d[a] = dw[a] * ds;
+            move[a] = fabsf(d[a]) >= 1.17549435e-38f;
+            if (!move[a]) {
+                // -(lo - o) in [0, size), decided exactly
+                const float s = -Ahi[a], e = -Alo[a];
                 const bool inside = (s > 0.f || (s == 0.f && e >= 0.f)) && (s < p.size || (s == p.size && e < 0.f));
                 if (!inside) return false;
-            } else {
-                df t0 = cross_time(0, h, Ahi[a], Alo[a], d[a], rd[a]);
-                df t1 = cross_time(R, h, Ahi[a], Alo[a], d[a], rd[a]);
-                if (d[a] < 0.f) {
-                    df tmp = t0;
-                    t0 = t1;
-                    t1 = tmp;
-                }
-                if (df_lt(tin, t0)) tin = t0;
-                if (df_lt(t1, tend)) tend = t1;
             }
+            Ahi[a] *= p.frame.ws;
+            Alo[a] *= p.frame.ws;
+            rd[a] = move[a] ? rcp_ftz(d[a]) : 0.f;
+            // the box's two planes: A / d and A / d + size / d
+            df t0, t1;
+            t0.hi = __fmul_rn(Ahi[a], rd[a]);
+            t0.lo = __fmul_rn(__fadd_rn(__fmaf_rn(-t0.hi, d[a], Ahi[a]), Alo[a]), rd[a]);
+            th[a] = __fmul_rn(p.frame.size, rd[a]);
+            tl[a] = __fmul_rn(__fmaf_rn(-th[a], d[a], p.frame.size), rd[a]);
+            float e;
+            two_sum(t0.hi, th[a], t1.hi, e);
+            t1.lo = __fadd_rn(e, __fadd_rn(t0.lo, tl[a]));
+            const bool neg = d[a] < 0.f;
+            const df t_in = neg ? t1 : t0, t_out = neg ? t0 : t1;
+            if (move[a] && df_lt(tin, t_in)) tin = t_in;
+            if (move[a] && df_lt(t_out, tend)) tend = t_out;
         }
         if (!df_lt(tin, tend)) return false;
-        // the unit of time: 2^-s, s from the exponent of the range
-        const int s = kTimeRangeExp + 127 - (int)(__float_as_uint(df_sub(tend, tin)) >> 23);
-        const float s1 = exp2_int(s / 2), s2 = exp2_int(s - s / 2);
-        unit = __fmul_rn(__fmul_rn(len, exp2_int(-(s / 2))), exp2_int(s / 2 - s));
-        tout = fixed_time(tend, tin, s1, s2);
+        tout = fixed_time_since(tend, tin);
         flip = 0;
         float rh[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            // error bound of the fp32 voxel-coordinate estimate, in voxels
-            const float margin = (fabsf(tend.hi * d[a]) + fabsf(Ahi[a])) * invh * 3.8146973e-6f + 1e-6f;
-            const int v = min(max(locate_axis(tin, d[a], Ahi[a], Alo[a], h, invh, margin), 0), R - 1);
             const bool neg = d[a] < 0.f;
-            q[a] = neg ? R - 1 - v : v;
             if (neg) flip |= 4u >> a;
-            nx[a] = hs[a] = kTimeNever;
-            if (d[a] != 0.f) {
-                nx[a] = fixed_time(cross_time(neg ? v : v + 1, h, Ahi[a], Alo[a], d[a], rd[a]), tin, s1, s2);
-                const float ard = fabsf(rd[a]), th = __fmul_rn(h, ard);
-                hs[a] = fixed_time({th, __fmul_rn(__fmaf_rn(-th, fabsf(d[a]), h), ard)}, {0.f, 0.f}, s1, s2);
+            // the voxel entered: an fp32 estimate low by its error bound, so exact or too low (by one unless
+            // the origin is far away), then exact tests of its upper plane's time (a point on a plane belongs
+            // to the voxel above)
+            const float g = __fmul_rn(__fmaf_rn(tin.hi, d[a], -Ahi[a]), invh);
+            const float margin = (fabsf(tin.hi * d[a]) + fabsf(Ahi[a])) * invh * 2.3841858e-7f + 1e-6f;
+            int v = min(max(__float2int_rd((neg ? (float)R - g : g) - margin), 0), R - 1);
+            hs[a] = fixed_time(fabsf(th[a]) * exp2_int(-p.depth), (neg ? -tl[a] : tl[a]) * exp2_int(-p.depth));
+            if (!move[a]) {
+                v = min(max(voxel_exact(o[a], p.lo[a], h / p.frame.ws, invh * p.frame.ws, R), 0), R - 1);
+                nx[a] = hs[a] = kTimeNever;
+            } else {
+                for (;; ++v) {
+                    nx[a] = fixed_time_since(cross_time(neg ? R - 1 - v : v + 1, h, Ahi[a], Alo[a], d[a], rd[a]), tin);
+                    if (nx[a] > 0 || v == R - 1) break;
+                }
             }
-            // planes per 2^20 units, a little below the true value (see cross_empty)
-            rh[a] = __fmul_rn(__fdividef(1048576.f, __ll2float_rn(hs[a])), 1.f - 9.5367432e-7f);
+            nx[a] = nx[a] < 0 ? 0 : nx[a];
+            q[a] = v;
+            // planes per 2^20 units, a little below the true value (see step)
+            rh[a] = fabsf(d[a]) * (invh * (exp2_int(20 - kTimeFrac) * (1.f - 9.5367432e-7f)));
         }
         *st = make_float4(rh[0], rh[1], rh[2], 0.f);
         // the mirror as an XOR mask: child slots (no index), entry offsets (dense), or brick offsets
         // with a flag per axis of the in-brick offset in bits 27-29 (brick layout)
-        if (p.cells) {
+        if (DENSE || BRICK || p.cells) {
             const uint32_t fx = flip & 4u ? R - 1 : 0, fy = flip & 2u ? R - 1 : 0, fz = flip & 1u ? R - 1 : 0;
-            const uint32_t bk = brick_of(fx, fy, fz, p.depth);
-            flip = p.btab ? bk | flip << 27 : (bk << 6) | in_brick(fx, fy, fz);
+            if (BRICK || (!DENSE && p.btab)) flip = brick_of(fx, fy, fz, p.depth) | flip << 27;
+            else flip = cell_index_offset(fx, fy, fz, p.depth);
         }
-        lvl_valid = 0;
-        if (!p.cells) stk[0] = 0;  // the stack exists only for trees without a cell index
+        if (!DENSE && !BRICK && !p.cells) stk[0] = stk[kMaxDepth * kBlock] = 0;  // the stack exists only for trees without a cell index
         cell = locate(p, stk, q);
         t = 0;
         step_i = 0;
         return true;
+    }
+
+    // The SH basis at the unit direction that begin() left in its row.
+    __device__ __forceinline__ void basis(const float u[3])
+    {
+        float Yt[K];
+        sh_basis<K>(u[0], u[1], u[2], Yt);
+        SmemY<K, kBlock>::store(ysm, Yt);
+    }
+
+    // One step of a lane in an empty box, its whole warp being in empty space:
+    // the box is crossed; false when the ray ends in it.
+    __device__ __forceinline__ bool approach(const RenderParams &p, int32_t *stk)
+    {
+        const int pq[3] = {q[0], q[1], q[2]};
+        t = leave_box();
+        if (t >= tout) return false;
+        if (step_i >= p.step_cap) {
+            *p.err = 1u;
+            return false;
+        }
+        ++step_i;
+        if ((unsigned)(q[0] | q[1] | q[2]) >= (unsigned)p.R) return false;
+        cell = locate(p, stk, pq);
+        return true;
+    }
+
+    // a4 for an empty box: the exit time, the earliest of its upper faces; every
+    // plane with a time <= it has then been crossed: floor((texit - nx) / hs) + 1
+    // of them per axis, by an fp32 estimate that is exact or one too low (its
+    // factor and its addend are low by 2^-20, over the rounding errors, and at
+    // most 2^12 planes are crossed), then the exact test of the next plane.
+    __device__ __forceinline__ int64_t leave_box()
+    {
+        const uint32_t m = cell & 0xFFFF, e = (cell >> 16) & 0xFF;
+        int64_t ex[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            ex[a] = nx[a] + (int64_t)((uint64_t)((m & ~(uint32_t)q[a]) + e) * (uint64_t)hs[a]);
+        const int64_t texit = min(ex[0], min(ex[1], ex[2]));
+        const float4 rh = *st;
+        const float r[3] = {rh.x, rh.y, rh.z};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const uint32_t c = __float2uint_rd(fmaf((float)(int)((texit - nx[a]) >> 20), r[a], 1.f - 9.5367432e-7f));
+            nx[a] += (int64_t)((uint64_t)c * (uint64_t)hs[a]);
+            q[a] += c;
+            if (nx[a] <= texit) {
+                nx[a] += hs[a];
+                ++q[a];
+            }
+        }
+        return texit;
     }
 
     template <typename Visitor>
@@ -249,27 +334,7 @@ struct Walker {
                 }
             }
         } else {
-            int64_t ex[3] = {nx[0], nx[1], nx[2]};
-            const uint32_t m = cell & 0xFFFF, e = (cell >> 16) & 0xFF;
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-                ex[a] += (int64_t)((uint64_t)((m & ~(uint32_t)q[a]) + e) * (uint64_t)hs[a]);
-            texit = min(ex[0], min(ex[1], ex[2]));
-            // planes crossed = floor((texit - nx) / hs) + 1, by an fp32 estimate that is exact or one too low
-            // (its factor and its addend are low by 2^-20, over the rounding errors, and at most 2^12 planes
-            // are crossed), then the exact test of the next plane
-            const float4 rh = *st;
-            const float r[3] = {rh.x, rh.y, rh.z};
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const uint32_t c = __float2uint_rd(fmaf((float)(int)((texit - nx[a]) >> 20), r[a], 1.f - 9.5367432e-7f));
-                nx[a] += (int64_t)((uint64_t)c * (uint64_t)hs[a]);
-                q[a] += c;
-                if (nx[a] <= texit) {
-                    nx[a] += hs[a];
-                    ++q[a];
-                }
-            }
+            texit = leave_box();
         }
         const bool last = texit >= tout, capped = !last && step_i >= p.step_cap;
         if (capped) *p.err = 1u;  // device error word: a plain store, no branch around an atomic
@@ -288,7 +353,7 @@ struct Walker {
 };
 
 // Per-thread scratch of a walk in shared memory: the SH basis (SmemY) and the
-// walker's row of per-axis constants, and the ancestor stack [kMaxDepth][kBlock] in
+// walker's row of constants, and the ancestor stack [kMaxDepth + 1][kBlock] in
 // dynamic shared memory, which a launch provides (walk_smem_bytes) only when
 // some tree of it has no cell index; without it the space goes to L1.
 // Declared once per kernel.
@@ -304,8 +369,19 @@ struct Walker {
 
 inline size_t walk_smem_bytes(bool need_stack)
 {
-    return need_stack ? sizeof(int32_t) * kMaxDepth * kBlock : 0;
+    return need_stack ? sizeof(int32_t) * (kMaxDepth + 1) * kBlock : 0;
 }
+
+// Whether a launch may use the kLookDense instance of a kernel that has no other than kLookAny.
+inline bool dense_index(const RenderParams &p) { return p.cells && !p.btab; }
+
+// FN<K, T, LOOKUP, ...> for the K of a tree; null for another K.
+#define POT_PICK_K(FN, K, T, LOOKUP, ...)                                                                       \
+    ((K) == 1 ? FN<1, T, LOOKUP, ##__VA_ARGS__> : (K) == 4 ? FN<4, T, LOOKUP, ##__VA_ARGS__>                    \
+     : (K) == 9 ? FN<9, T, LOOKUP, ##__VA_ARGS__> : (K) == 16 ? FN<16, T, LOOKUP, ##__VA_ARGS__>                \
+     : (K) == 25 ? FN<25, T, LOOKUP, ##__VA_ARGS__> : nullptr)
+#define POT_PICK_WALK(FN, K, T, DENSE, ...)                                                                     \
+    ((DENSE) ? POT_PICK_K(FN, K, T, kLookDense, ##__VA_ARGS__) : POT_PICK_K(FN, K, T, kLookAny, ##__VA_ARGS__))
 
 // Grid of a persistent walk kernel: one wave of resident blocks (SMs x blocks
 // per SM for this kernel and shared memory), no more blocks than tiles need.
@@ -326,22 +402,40 @@ cudaError_t persistent_grid(Fn fn, size_t smem, int64_t n_tiles, int max_blocks,
     return cudaSuccess;
 }
 
-// The whole walk of one ray.
-template <int K, typename T, typename Visitor>
-__device__ __forceinline__ void walk_ray(const RenderParams &p, int32_t *stk, float *ysm, float4 *wst,
-                                         const float o[3], const float d[3], float near, float far, Visitor &vis)
+// The walks of a warp's 32 rays (every lane calls it; has: whether it has a
+// ray).  APPROACH (tiles of pixels, whose rays meet the scene together): while
+// no lane has met a leaf the warp crosses empty space in a loop of its own,
+// without the leaf side of step(), and the SH basis is evaluated once some lane
+// has, so tiles that see no leaf never do.
+template <int K, typename T, Lookup LOOKUP, bool APPROACH, typename Visitor>
+__device__ __forceinline__ void walk_rays(const RenderParams &p, int32_t *stk, float *ysm, float4 *wst, bool has,
+                                          const float o[3], const float d[3], float near, float far, Visitor &vis)
 {
-    Walker<K, T> w;
+    Walker<K, T, LOOKUP> w;
     w.ysm = ysm;
     w.st = wst;
-    if (!w.begin(p, stk, o, d, near, far)) return;
-    while (w.step(p, stk, vis)) {
+    float u[3] = {0.f, 0.f, 1.f};
+    has = has && w.begin(p, stk, o, d, near, far, u);
+    if (APPROACH) {
+        while (!__any_sync(0xffffffffu, has && w.cell >= 0)) {
+            if (has) has = w.approach(p, stk);
+            if (!__any_sync(0xffffffffu, has)) return;
+        }
+    }
+    if (Visitor::kBasis && has) w.basis(u);
+    if (Visitor::kVote) {
+        while (__any_sync(0xffffffffu, has)) {
+            if (has) has = w.step(p, stk, vis);
+        }
+    } else {
+        while (has) has = w.step(p, stk, vis);
     }
 }
 
 // a5-a8 for one leaf segment: fetch, colour, composite, early stop.
 template <int K, typename T, bool COUNT>
 struct ShadeVisitor {
+    static constexpr bool kBasis = true, kVote = false;
     const T *sig_arr;
     const T *sh_arr;
     uint8_t *touched;
@@ -385,12 +479,12 @@ __device__ __forceinline__ bool tile_ray(const RenderParams &p, unsigned long lo
         const uint32_t tl = (uint32_t)tile;
         const uint32_t G = (uint32_t)p.view_group;
         const uint32_t per_group = (uint32_t)p.tiles_per_cam * G;
-        const uint32_t group = tl / per_group;
+        const uint32_t group = p.by_group(tl);
         const uint32_t in_group = tl - group * per_group;
         const uint32_t gsize = min(G, (uint32_t)p.n_cams - group * G);
-        const int64_t cam = (int64_t)(group * G + in_group % gsize);
-        const uint32_t rem = in_group / gsize;
-        const int ty = (int)(rem / (uint32_t)p.tiles_x);
+        const uint32_t rem = gsize == G ? p.by_view(in_group) : p.by_last(in_group);
+        const int64_t cam = (int64_t)(group * G + in_group - rem * gsize);
+        const int ty = (int)p.by_row(rem);
         const int tx = (int)(rem - (uint32_t)ty * (uint32_t)p.tiles_x);
         const int i = tx * kTileW + (slot % kTileW);
         const int j = ty * kTileH + (slot / kTileW);
@@ -432,8 +526,8 @@ __device__ __forceinline__ void store_ray(const RenderParams &p, int64_t ray, co
 
 // Forward render, one tile per warp at a time: the warp takes the next tile
 // once all 32 of its rays are done.
-template <int K, typename T, bool CAMS, bool COUNT>
-__global__ void __launch_bounds__(kBlock, POT_RENDER_MIN_BLOCKS) render_kernel(const RenderParams p)
+template <int K, typename T, Lookup LOOKUP, bool CAMS, bool COUNT>
+__global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) render_kernel(const RenderParams p)
 {
     POT_WALK_SHARED(K)
     const int lane = threadIdx.x & 31;
@@ -446,12 +540,10 @@ __global__ void __launch_bounds__(kBlock, POT_RENDER_MIN_BLOCKS) render_kernel(c
         if (tile >= (unsigned long long)p.n_tiles) break;
         float o[3], d[3], near, far;
         int64_t ray;
-        if (tile_ray<CAMS>(p, tile, lane, o, d, near, far, ray)) {
-            ShadeVisitor<K, T, COUNT> v{sig_arr, sh_arr, p.leaf_touched, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0,
-                                        p.codebook};
-            walk_ray<K, T>(p, stk, ysm, wst, o, d, near, far, v);
-            store_ray<K, T, COUNT>(p, ray, v);
-        }
+        const bool has = tile_ray<CAMS>(p, tile, lane, o, d, near, far, ray);
+        ShadeVisitor<K, T, COUNT> v{sig_arr, sh_arr, p.leaf_touched, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, p.codebook};
+        walk_rays<K, T, LOOKUP, CAMS>(p, stk, ysm, wst, has, o, d, near, far, v);
+        if (has) store_ray<K, T, COUNT>(p, ray, v);
     }
 }
 
@@ -461,10 +553,17 @@ cudaError_t launch_render_t(const RenderParams &p, int K, bool cams, bool count,
 {
     using Fn = void (*)(const RenderParams);
     Fn fn = nullptr;
-#define POT_PICK(KK)                                                                            \
-    if (K == KK)                                                                                \
-        fn = cams ? (count ? render_kernel<KK, T, true, true> : render_kernel<KK, T, true, false>) \
-                  : (count ? render_kernel<KK, T, false, true> : render_kernel<KK, T, false, false>);
+    // counting launches (measurement) and explicit rays have fewer instances of their own
+    const Lookup look = p.btab ? kLookBrick : p.cells ? kLookDense : kLookAny;
+#define POT_PICK(KK)                                                                  \
+    if (K == KK)                                                                      \
+        fn = cams ? (count                ? render_kernel<KK, T, kLookAny, true, true>   \
+                     : look == kLookDense ? render_kernel<KK, T, kLookDense, true, false> \
+                     : look == kLookBrick ? render_kernel<KK, T, kLookBrick, true, false> \
+                                          : render_kernel<KK, T, kLookAny, true, false>)  \
+                  : (count                ? render_kernel<KK, T, kLookAny, false, true>   \
+                     : look == kLookDense ? render_kernel<KK, T, kLookDense, false, false> \
+                                          : render_kernel<KK, T, kLookAny, false, false>);
     POT_PICK(1)
     POT_PICK(4)
     POT_PICK(9)
@@ -476,7 +575,9 @@ cudaError_t launch_render_t(const RenderParams &p, int K, bool cams, bool count,
     unsigned grid = 0;
     cudaError_t e = persistent_grid(fn, smem, p.n_tiles, max_blocks, &grid);
     if (e != cudaSuccess) return e;
-    fn<<<grid, kBlock, smem, s>>>(p);
+    RenderParams q = p;
+    if (cams) set_tile_divs(q);
+    fn<<<grid, kBlock, smem, s>>>(q);
     count_launch();
     return cudaGetLastError();
 }
