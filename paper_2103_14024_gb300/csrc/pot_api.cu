@@ -53,6 +53,19 @@ WalkFrame walk_frame(float size, int depth)
     return f;
 }
 
+bool one_wave(int64_t n_tiles)
+{
+    static std::atomic<int> sms[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    int n = sms[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+        sms[dev].store(n, std::memory_order_relaxed);
+    }
+    return n_tiles <= 16ll * n;
+}
+
 int render_view_group(int n_cams)
 {
     static int g = [] {
@@ -158,6 +171,33 @@ struct Tmp {
         return cudaMallocFromPoolAsync(&p, bytes > 0 ? bytes : 16, pool, st);
     }
 };
+
+// What a walk launch needs on the device besides its arrays: tile counters
+// (zeroed; none where one wave of warps takes all tiles) and the cameras (none
+// where they fit into the launch).  Both in one buffer and one copy.
+cudaError_t walk_scratch(RenderParams &p, Tmp &mem, const pot_camera *cams, int n_cams, int n_counters, bool few_ok,
+                         cudaStream_t s)
+{
+    const bool few = n_cams <= kFewCams && few_ok;
+    if (n_cams > 0 && few) std::memcpy(p.few_cams, cams, sizeof(pot_camera) * n_cams);
+    const size_t cam_bytes = few ? 0 : sizeof(pot_camera) * (size_t)n_cams;
+    const size_t cnt_bytes = n_counters ? (sizeof(unsigned long long) * (size_t)n_counters + 255) / 256 * 256 : 0;
+    if (cnt_bytes + cam_bytes == 0) return cudaSuccess;
+    cudaError_t e = mem.alloc(cnt_bytes + cam_bytes, s);
+    if (e != cudaSuccess) return e;
+    char *d = static_cast<char *>(mem.p);
+    if (n_counters) p.tile_counter = reinterpret_cast<unsigned long long *>(d);
+    if (cam_bytes) p.cams = reinterpret_cast<const pot_camera *>(d + cnt_bytes);
+    char h[20480];  // 200 cameras and their counters fit
+    if (cam_bytes && cnt_bytes + cam_bytes <= sizeof(h)) {
+        std::memset(h, 0, cnt_bytes);
+        std::memcpy(h + cnt_bytes, cams, cam_bytes);
+        return cudaMemcpyAsync(d, h, cnt_bytes + cam_bytes, cudaMemcpyHostToDevice, s);  // staged before it returns
+    }
+    if (cnt_bytes) e = cudaMemsetAsync(d, 0, cnt_bytes, s);
+    if (e == cudaSuccess && cam_bytes) e = cudaMemcpyAsync(d + cnt_bytes, cams, cam_bytes, cudaMemcpyHostToDevice, s);
+    return e;
+}
 
 // A device view of an input array that may live in host memory.
 cudaError_t stage_in(const void *src, size_t bytes, Tmp &tmp, cudaStream_t s, const void **out)
@@ -386,10 +426,10 @@ cudaError_t launch_render(const RenderParams &p, const pot_tree *t, bool cams, c
 {
     const bool count = p.seg_count != nullptr;
     switch (t->desc.leaf_dtype) {
-    case POT_F32: return launch_render_f32(p, t->K, cams, count, s, 0);
-    case POT_F16: return launch_render_f16(p, t->K, cams, count, s, 0);
-    case POT_CB16: return launch_render_cb16(p, t->K, cams, count, s, 0);
-    default: return launch_render_bf16(p, t->K, cams, count, s, 0);
+    case POT_F32: return launch_render_f32(p, t->K, cams, count, s);
+    case POT_F16: return launch_render_f16(p, t->K, cams, count, s);
+    case POT_CB16: return launch_render_cb16(p, t->K, cams, count, s);
+    default: return launch_render_bf16(p, t->K, cams, count, s);
     }
 }
 
@@ -757,15 +797,7 @@ pot_status pot_render(const pot_tree *t, const pot_camera *cams, int32_t n_cams,
     }
     DeviceGuard g(t->device);
     cudaStream_t s = (cudaStream_t)stream;
-    const int64_t npix = (int64_t)n_cams * W * H;
     Tmp scratch;
-    // tile counters (one per launch: a host-memory output renders in chunks), then the cameras
-    const size_t cam_off = ((sizeof(unsigned long long) * (size_t)(n_cams + 1) + 255) / 256) * 256;
-    POT_CUDA(scratch.alloc(cam_off + sizeof(pot_camera) * n_cams, s), "alloc scratch");
-    char *sp = static_cast<char *>(scratch.p);
-    POT_CUDA(cudaMemsetAsync(sp, 0, cam_off, s), "memset");
-    POT_CUDA(cudaMemcpyAsync(sp + cam_off, cams, sizeof(pot_camera) * n_cams, cudaMemcpyHostToDevice, s),
-             "copy cams");
     RenderParams p;
     fill_tree_params(p, t, opts);
     if (!p.err) return fail(POT_ERR_CUDA, "device error word unavailable");
@@ -775,18 +807,17 @@ pot_status pot_render(const pot_tree *t, const pot_camera *cams, int32_t n_cams,
     p.tiles_per_cam = (int64_t)p.tiles_x * ((H + kTileH - 1) / kTileH);
     if (p.tiles_per_cam * ((int64_t)n_cams + 16) >= (1ll << 32))
         return tile_limit_error();
-    p.tile_counter = reinterpret_cast<unsigned long long *>(sp);
-    const pot_camera *d_cams = reinterpret_cast<const pot_camera *>(sp + cam_off);
     const bool host_out = !is_device_ptr(rgb) || (t_final && !is_device_ptr(t_final));
-    if (host_out) return render_to_host(p, t, d_cams, n_cams, rgb, t_final, s);
-    p.cams = d_cams;
+    p.n_tiles = p.tiles_per_cam * n_cams;
+    // a host-memory output renders in chunks, one counter each
+    const int n_counters = host_out ? n_cams : one_wave(p.n_tiles) ? 0 : 1;
+    POT_CUDA(walk_scratch(p, scratch, cams, n_cams, n_counters, !host_out, s), "scratch");
+    if (host_out) return render_to_host(p, t, p.cams, n_cams, rgb, t_final, s);
     p.n_cams = n_cams;
     p.view_group = render_view_group(n_cams);
-    p.n_tiles = p.tiles_per_cam * n_cams;
     p.rgb = rgb;
     p.t_final = t_final;
     POT_CUDA(launch_render(p, t, true, s), "render");
-    (void)npix;
     return POT_OK;
 }
 
@@ -807,8 +838,6 @@ pot_status pot_render_rays(const pot_tree *t, int64_t n, const float *origins, c
     const void *dor, *ddr;
     POT_CUDA(stage_in(origins, sizeof(float) * 3 * n, to, s, &dor), "stage origins");
     POT_CUDA(stage_in(dirs, sizeof(float) * 3 * n, td, s, &ddr), "stage dirs");
-    POT_CUDA(scratch.alloc(sizeof(unsigned long long), s), "alloc scratch");
-    POT_CUDA(cudaMemsetAsync(scratch.p, 0, sizeof(unsigned long long), s), "memset");
     Out orgb, otf;
     void *drgb, *dtf = nullptr;
     POT_CUDA(orgb.bind(rgb, sizeof(float) * 3 * n, s, &drgb), "bind rgb");
@@ -824,7 +853,7 @@ pot_status pot_render_rays(const pot_tree *t, int64_t n, const float *origins, c
     p.n_tiles = (n + 31) / 32;
     p.rgb = (float *)drgb;
     p.t_final = (float *)dtf;
-    p.tile_counter = static_cast<unsigned long long *>(scratch.p);
+    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles) ? 0 : 1, true, s), "scratch");
     POT_CUDA(launch_render(p, t, false, s), "render_rays");
     POT_CUDA(orgb.finish(s), "copy rgb");
     POT_CUDA(otf.finish(s), "copy t_final");
@@ -852,15 +881,9 @@ pot_status pot_visibility(const pot_tree *t, const pot_camera *cams, int32_t n_c
     DeviceGuard g(t->device);
     cudaStream_t s = (cudaStream_t)stream;
     Tmp scratch;
-    const size_t cam_off = 256;
-    POT_CUDA(scratch.alloc(cam_off + sizeof(pot_camera) * n_cams, s), "alloc scratch");
-    char *sp = static_cast<char *>(scratch.p);
-    POT_CUDA(cudaMemsetAsync(sp, 0, cam_off, s), "memset");
-    POT_CUDA(cudaMemcpyAsync(sp + cam_off, cams, sizeof(pot_camera) * n_cams, cudaMemcpyHostToDevice, s), "copy cams");
     RenderParams p;
     fill_tree_params(p, t, opts);
     if (!p.err) return fail(POT_ERR_CUDA, "device error word unavailable");
-    p.cams = reinterpret_cast<const pot_camera *>(sp + cam_off);
     p.n_cams = n_cams;
     p.view_group = render_view_group(n_cams);
     p.W = W;
@@ -870,7 +893,7 @@ pot_status pot_visibility(const pot_tree *t, const pot_camera *cams, int32_t n_c
     if (p.tiles_per_cam * ((int64_t)n_cams + 16) >= (1ll << 32))
         return tile_limit_error();
     p.n_tiles = p.tiles_per_cam * n_cams;
-    p.tile_counter = reinterpret_cast<unsigned long long *>(sp);
+    POT_CUDA(walk_scratch(p, scratch, cams, n_cams, one_wave(p.n_tiles) ? 0 : 1, true, s), "scratch");
     POT_CUDA(launch_visibility(p, t, max_weight, s), "visibility");
     return POT_OK;
 }
@@ -998,8 +1021,6 @@ pot_status pot_render_backward(const pot_tree *t, int64_t n, const float *origin
     DeviceGuard g(t->device);
     cudaStream_t s = (cudaStream_t)stream;
     Tmp scratch;
-    POT_CUDA(scratch.alloc(sizeof(unsigned long long), s), "alloc scratch");
-    POT_CUDA(cudaMemsetAsync(scratch.p, 0, sizeof(unsigned long long), s), "memset");
     RenderParams p;
     fill_tree_params(p, t, opts);
     if (!p.err) return fail(POT_ERR_CUDA, "device error word unavailable");
@@ -1009,7 +1030,7 @@ pot_status pot_render_backward(const pot_tree *t, int64_t n, const float *origin
     p.near = near;
     p.far = far;
     p.n_tiles = (n + 31) / 32;
-    p.tile_counter = static_cast<unsigned long long *>(scratch.p);
+    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles) ? 0 : 1, true, s), "scratch");
     POT_CUDA(launch_backward(p, grad_rgb, rgb_fwd, grad_sigma, grad_sh, t->desc.leaf_dtype, t->K, s), "backward");
     return POT_OK;
 }
@@ -1038,8 +1059,6 @@ pot_status pot_render_mse_backward(const pot_tree *t, int64_t n, const float *or
     DeviceGuard g(t->device);
     cudaStream_t s = (cudaStream_t)stream;
     Tmp scratch;
-    POT_CUDA(scratch.alloc(sizeof(unsigned long long), s), "alloc scratch");
-    POT_CUDA(cudaMemsetAsync(scratch.p, 0, sizeof(unsigned long long), s), "memset");
     POT_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), s), "memset loss");
     RenderParams p;
     fill_tree_params(p, t, opts);
@@ -1050,7 +1069,7 @@ pot_status pot_render_mse_backward(const pot_tree *t, int64_t n, const float *or
     p.near = near;
     p.far = far;
     p.n_tiles = (n + 31) / 32;
-    p.tile_counter = static_cast<unsigned long long *>(scratch.p);
+    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles) ? 0 : 1, true, s), "scratch");
     POT_CUDA(launch_mse_backward(p, target, rgb, loss, grad_sigma, grad_sh, t->desc.leaf_dtype, t->K, s),
              "mse backward");
     return POT_OK;
@@ -1095,8 +1114,6 @@ pot_status pot_render_rays_record(const pot_tree *t, int64_t n, const float *ori
     POT_CUDA(cudaMemsetAsync(seg_state, 0, 2 * sizeof(int64_t), s), "clear seg_state");
     if (n == 0) return POT_OK;
     Tmp scratch;
-    POT_CUDA(scratch.alloc(sizeof(unsigned long long), s), "alloc scratch");
-    POT_CUDA(cudaMemsetAsync(scratch.p, 0, sizeof(unsigned long long), s), "memset");
     RenderParams p;
     fill_tree_params(p, t, opts);
     if (!p.err) return fail(POT_ERR_CUDA, "device error word unavailable");
@@ -1108,7 +1125,7 @@ pot_status pot_render_rays_record(const pot_tree *t, int64_t n, const float *ori
     p.n_tiles = (n + 31) / 32;
     p.rgb = rgb;
     p.t_final = t_final;
-    p.tile_counter = static_cast<unsigned long long *>(scratch.p);
+    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles) ? 0 : 1, true, s), "scratch");
     const SegmentBuffer sb{static_cast<float4 *>(records), capacity, reinterpret_cast<unsigned long long *>(seg_state)};
     POT_CUDA(launch_render_record(p, sb, t->desc.leaf_dtype, t->K, s), "render_rays_record");
     return POT_OK;
@@ -1139,8 +1156,6 @@ pot_status pot_render_backward_recorded(const pot_tree *t, int64_t n, const floa
     DeviceGuard g(t->device);
     cudaStream_t s = (cudaStream_t)stream;
     Tmp scratch;  // tile counter of the walking fallback
-    POT_CUDA(scratch.alloc(sizeof(unsigned long long), s), "alloc scratch");
-    POT_CUDA(cudaMemsetAsync(scratch.p, 0, sizeof(unsigned long long), s), "memset");
     RenderParams p;
     fill_tree_params(p, t, opts);
     if (!p.err) return fail(POT_ERR_CUDA, "device error word unavailable");
@@ -1150,7 +1165,7 @@ pot_status pot_render_backward_recorded(const pot_tree *t, int64_t n, const floa
     p.near = near;
     p.far = far;
     p.n_tiles = (n + 31) / 32;
-    p.tile_counter = static_cast<unsigned long long *>(scratch.p);
+    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles) ? 0 : 1, true, s), "scratch");
     const SegmentBuffer sb{static_cast<float4 *>(const_cast<void *>(records)), capacity,
                            reinterpret_cast<unsigned long long *>(const_cast<int64_t *>(seg_state))};
     // scratch of the bin order: bins of 2^bb leaves (count, start, cursor)

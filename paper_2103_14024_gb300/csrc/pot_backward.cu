@@ -176,7 +176,7 @@ enum BackwardMode { kGradAndColour = 0, kGrad = 1, kMseTarget = 2 };
 // walk; kMseTarget: C from a first walk, then dL/dC of the MSE against the
 // target, the loss summed per warp into *loss, C optionally written out.
 template <int K, typename T, Lookup LOOKUP, int MODE>
-__global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kernel(const BackwardParams bp)
+__global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kernel(const __grid_constant__ BackwardParams bp)
 {
     POT_WALK_SHARED(K)
     const RenderParams &p = bp.r;
@@ -184,11 +184,8 @@ __global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kern
     const int lane = threadIdx.x & 31;
     const T *sig_arr = static_cast<const T *>(p.sigma);
     const T *sh_arr = static_cast<const T *>(p.sh);
-    for (;;) {
-        unsigned long long tile = 0;
-        if (lane == 0) tile = atomicAdd(p.tile_counter, 1ull);
-        tile = __shfl_sync(0xffffffffu, tile, 0);
-        if (tile >= (unsigned long long)p.n_tiles) break;
+    int taken = 0;
+    for (unsigned long long tile; next_tile(p, lane, taken, tile);) {
         const int64_t ray = (int64_t)tile * 32 + lane;
         float lsum = 0.f;  // this ray's squared error (MSE mode)
         const bool has = ray < p.n_rays;
@@ -255,7 +252,7 @@ cudaError_t launch_backward_t(const BackwardParams &bp, int K, int mode, cudaStr
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = walk_smem_bytes(bp.r.cells == nullptr);
     unsigned grid = 0;
-    cudaError_t e = persistent_grid(fn, smem, bp.r.n_tiles, 0, &grid);
+    cudaError_t e = persistent_grid(fn, smem, bp.r.n_tiles, bp.r.tile_counter, &grid);
     if (e != cudaSuccess) return e;
     fn<<<grid, kBlock, smem, s>>>(bp);
     count_launch();

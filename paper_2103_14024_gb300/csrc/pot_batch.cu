@@ -40,7 +40,6 @@ struct BatchParams {
     const BatchItem *items;
     int n_items;
     int64_t n_tiles;
-    unsigned long long *tile_counter;
     unsigned int *err;
 };
 
@@ -133,7 +132,7 @@ cudaError_t launch_batch_t(const BatchParams &bp, int K, Lookup look, bool need_
 }  // namespace
 
 // items: host array of n validated requests; groups by (K, dtype, cell index), stages the
-// descriptors and one counter per group in a single stream-ordered buffer.
+// descriptors in a stream-ordered buffer.
 cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_t s, unsigned int *err)
 {
     std::vector<int> order(n);
@@ -179,17 +178,13 @@ cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_
     }
     group_start.push_back(n);
     const int groups = (int)group_start.size() - 1;
-    const size_t cnt_bytes = 256;
-    const size_t bytes = cnt_bytes + sizeof(BatchItem) * (size_t)n;
-    void *buf = nullptr;
+    BatchItem *d_items = nullptr;
     cudaMemPool_t pool = nullptr;
     cudaError_t e = scratch_pool(&pool);
-    if (e == cudaSuccess) e = cudaMallocFromPoolAsync(&buf, bytes, pool, s);
+    if (e == cudaSuccess)
+        e = cudaMallocFromPoolAsync(reinterpret_cast<void **>(&d_items), sizeof(BatchItem) * (size_t)n, pool, s);
     if (e != cudaSuccess) return e;
-    char *cb = static_cast<char *>(buf);
-    BatchItem *d_items = reinterpret_cast<BatchItem *>(cb + cnt_bytes);
-    e = cudaMemsetAsync(cb, 0, cnt_bytes, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d_items, desc.data(), sizeof(BatchItem) * n, cudaMemcpyHostToDevice, s);
+    e = cudaMemcpyAsync(d_items, desc.data(), sizeof(BatchItem) * n, cudaMemcpyHostToDevice, s);
     for (int g = 0; g < groups && e == cudaSuccess; ++g) {
         const int a = group_start[g], b = group_start[g + 1];
         const BatchItem &last = desc[b - 1];
@@ -197,7 +192,6 @@ cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_
         bp.items = d_items + a;
         bp.n_items = b - a;
         bp.n_tiles = last.tile_begin + (int64_t)last.tiles_x * ((last.H + kTileH - 1) / kTileH);
-        bp.tile_counter = reinterpret_cast<unsigned long long *>(cb) + g;
         bp.err = err;
         const pot_tree *t = items[order[a]].tree;
         const Lookup look = t->cell_kind == POT_CELLS_DENSE   ? kLookDense
@@ -211,7 +205,7 @@ cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_
         default: e = launch_batch_t<__nv_bfloat16>(bp, t->K, look, need_stack, s); break;
         }
     }
-    cudaFreeAsync(buf, s);
+    cudaFreeAsync(d_items, s);
     return e;
 }
 

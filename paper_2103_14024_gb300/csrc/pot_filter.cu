@@ -30,16 +30,13 @@ struct MaxWeightVisitor {
 };
 
 template <int K, typename T, Lookup LOOKUP>
-__global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) visibility_kernel(const RenderParams p, float *max_w)
+__global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) visibility_kernel(const __grid_constant__ RenderParams p, float *max_w)
 {
     POT_WALK_SHARED(K)
     const int lane = threadIdx.x & 31;
     const T *sig_arr = static_cast<const T *>(p.sigma);
-    for (;;) {
-        unsigned long long tile = 0;
-        if (lane == 0) tile = atomicAdd(p.tile_counter, 1ull);
-        tile = __shfl_sync(0xffffffffu, tile, 0);
-        if (tile >= (unsigned long long)p.n_tiles) break;
+    int taken = 0;
+    for (unsigned long long tile; next_tile(p, lane, taken, tile);) {
         float o[3], d[3], near, far;
         int64_t ray;
         const bool has = tile_ray<true>(p, tile, lane, o, d, near, far, ray);
@@ -56,7 +53,7 @@ cudaError_t launch_visibility_t(const RenderParams &p, int K, float *max_w, cuda
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = walk_smem_bytes(p.cells == nullptr);
     unsigned grid = 0;
-    cudaError_t e = persistent_grid(fn, smem, p.n_tiles, 0, &grid);
+    cudaError_t e = persistent_grid(fn, smem, p.n_tiles, p.tile_counter, &grid);
     if (e != cudaSuccess) return e;
     RenderParams q = p;
     set_tile_divs(q);

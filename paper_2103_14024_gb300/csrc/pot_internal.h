@@ -73,6 +73,8 @@ struct WalkFrame {
 constexpr int kTimeFrac = 49;
 WalkFrame walk_frame(float size, int depth);
 
+constexpr int kFewCams = 8;  // 640 bytes of launch parameters
+
 // Everything a render launch needs; passed by value.
 struct RenderParams {
     const int32_t *child;
@@ -90,7 +92,7 @@ struct RenderParams {
     float gamma;
     int step_cap;
     // ray source: cameras (tiles of kTileW x kTileH pixels) or explicit rays (32 per tile)
-    const pot_camera *cams;
+    const pot_camera *cams;  // null: the first n_cams of few_cams
     int n_cams;
     int view_group;     // tiles are interleaved over groups of this many consecutive cameras
     int W, H;
@@ -108,8 +110,11 @@ struct RenderParams {
     int32_t *seg_count;
     uint8_t *leaf_touched;
     // scratch
-    unsigned long long *tile_counter;
+    unsigned long long *tile_counter;  // null: one tile per warp, in order
     unsigned int *err;
+    // cameras of calls with few of them: they travel in the launch instead of
+    // a copy of their own ahead of it
+    pot_camera few_cams[kFewCams];
 };
 
 // The divisors of tile numbers, from the camera fields (view_group, n_cams, tiles).
@@ -123,14 +128,10 @@ inline void set_tile_divs(RenderParams &p)
 }
 
 // Launches (defined in pot_render_*.cu); return the CUDA error of the launch.
-cudaError_t launch_render_f32(const RenderParams &p, int K, bool cams, bool count, cudaStream_t s,
-                              int max_blocks);
-cudaError_t launch_render_f16(const RenderParams &p, int K, bool cams, bool count, cudaStream_t s,
-                              int max_blocks);
-cudaError_t launch_render_bf16(const RenderParams &p, int K, bool cams, bool count, cudaStream_t s,
-                               int max_blocks);
-cudaError_t launch_render_cb16(const RenderParams &p, int K, bool cams, bool count, cudaStream_t s,
-                               int max_blocks);
+cudaError_t launch_render_f32(const RenderParams &p, int K, bool cams, bool count, cudaStream_t s);
+cudaError_t launch_render_f16(const RenderParams &p, int K, bool cams, bool count, cudaStream_t s);
+cudaError_t launch_render_bf16(const RenderParams &p, int K, bool cams, bool count, cudaStream_t s);
+cudaError_t launch_render_cb16(const RenderParams &p, int K, bool cams, bool count, cudaStream_t s);
 
 // Build / query / export helpers (pot_build.cu, pot_query.cu).
 cudaError_t build_levels_and_children(pot_tree *t, int64_t n, const uint64_t *d_codes, cudaStream_t s,
@@ -164,6 +165,12 @@ cudaError_t compact_kept_leaves(const pot_tree *t, const float *score, float thr
                                 float **sig_out, float **sh_out, int64_t *n_keep, cudaStream_t s);
 cudaError_t quantize_tree(const pot_tree *t, int bits, pot_tree *q, cudaStream_t s);
 cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_t s, unsigned int *err);
+
+// Whether n_tiles tiles are all resident at once in every walk kernel (16 warps
+// per SM at least): then warp i takes tile i, and the launch needs no tile
+// counter, that is no allocation and no memset before it.  (With the cameras in
+// the launch too, one 256 x 256 view 88 -> 77 us, one 64 x 64 view 26 -> 23 us.)
+bool one_wave(int64_t n_tiles);
 
 // cameras interleaved per tile group in camera renders (POT_VIEW_GROUP overrides)
 int render_view_group(int n_cams);

@@ -199,10 +199,10 @@ pot_status pot_render_noalloc(const pot_tree *t, const pot_camera *cams, int32_t
     p.tile_counter = reinterpret_cast<unsigned long long *>(scratch);
     const bool count = p.seg_count != nullptr;
     switch (t->desc.leaf_dtype) {
-    case POT_F32: e = launch_render_f32(p, t->K, true, count, s, 0); break;
-    case POT_F16: e = launch_render_f16(p, t->K, true, count, s, 0); break;
-    case POT_CB16: e = launch_render_cb16(p, t->K, true, count, s, 0); break;
-    default: e = launch_render_bf16(p, t->K, true, count, s, 0); break;
+    case POT_F32: e = launch_render_f32(p, t->K, true, count, s); break;
+    case POT_F16: e = launch_render_f16(p, t->K, true, count, s); break;
+    case POT_CB16: e = launch_render_cb16(p, t->K, true, count, s); break;
+    default: e = launch_render_bf16(p, t->K, true, count, s); break;
     }
     if (e != cudaSuccess) return na_cuda(e, "render launch");
     return POT_OK;

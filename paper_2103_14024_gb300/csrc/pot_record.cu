@@ -44,7 +44,7 @@ struct RecordVisitor {
 
 template <int K, typename T, Lookup LOOKUP>
 __global__ void __launch_bounds__(kBlock, POT_RECORD_MIN_BLOCKS)
-    record_kernel(const RenderParams p, const SegmentBuffer sb)
+    record_kernel(const __grid_constant__ RenderParams p, const SegmentBuffer sb)
 {
     POT_WALK_SHARED(K)
     const int lane = threadIdx.x & 31;
@@ -57,11 +57,8 @@ __global__ void __launch_bounds__(kBlock, POT_RECORD_MIN_BLOCKS)
     long long base = -1;
     int fill = kSegBlock;
     bool dead = false;
-    for (;;) {
-        unsigned long long tile = 0;
-        if (lane == 0) tile = atomicAdd(p.tile_counter, 1ull);
-        tile = __shfl_sync(0xffffffffu, tile, 0);
-        if (tile >= (unsigned long long)p.n_tiles) break;
+    int taken = 0;
+    for (unsigned long long tile; next_tile(p, lane, taken, tile);) {
         const int64_t ray = (int64_t)tile * 32 + lane;
         RecordVisitor<K, T> v;
         v.sv = ShadeVisitor<K, T, false>{sig_arr, sh_arr, nullptr, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, nullptr};
@@ -132,7 +129,7 @@ cudaError_t launch_record_t(const RenderParams &p, const SegmentBuffer &sb, int 
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = walk_smem_bytes(p.cells == nullptr);
     unsigned grid = 0;
-    cudaError_t e = persistent_grid(fn, smem, p.n_tiles, 0, &grid);
+    cudaError_t e = persistent_grid(fn, smem, p.n_tiles, p.tile_counter, &grid);
     if (e != cudaSuccess) return e;
     fn<<<grid, kBlock, smem, s>>>(p, sb);
     count_launch();

@@ -383,20 +383,40 @@ inline bool dense_index(const RenderParams &p) { return p.cells && !p.btab; }
 #define POT_PICK_WALK(FN, K, T, DENSE, ...)                                                                     \
     ((DENSE) ? POT_PICK_K(FN, K, T, kLookDense, ##__VA_ARGS__) : POT_PICK_K(FN, K, T, kLookAny, ##__VA_ARGS__))
 
-// Grid of a persistent walk kernel: one wave of resident blocks (SMs x blocks
+// The next tile of a warp: from the launch's counter until none is left, or,
+// without one, the tile of the warp's place in the grid, once (taken counts the
+// calls).  False when there is none.
+__device__ __forceinline__ bool next_tile(const RenderParams &p, int lane, int &taken, unsigned long long &tile)
+{
+    if (p.tile_counter) {
+        tile = 0;
+        if (lane == 0) tile = atomicAdd(p.tile_counter, 1ull);
+        tile = __shfl_sync(0xffffffffu, tile, 0);
+    } else {
+        if (taken++) return false;
+        tile = (unsigned long long)blockIdx.x * (kBlock / 32) + (threadIdx.x >> 5);
+    }
+    return tile < (unsigned long long)p.n_tiles;
+}
+
+// Grid of a walk kernel: a block per kBlock / 32 tiles where every warp takes one
+// (counter null), else one wave of resident blocks (SMs x blocks
 // per SM for this kernel and shared memory), no more blocks than tiles need.
 template <typename Fn>
-cudaError_t persistent_grid(Fn fn, size_t smem, int64_t n_tiles, int max_blocks, unsigned *grid)
+cudaError_t persistent_grid(Fn fn, size_t smem, int64_t n_tiles, const void *counter, unsigned *grid)
 {
+    const int64_t need = (n_tiles + (kBlock / 32) - 1) / (kBlock / 32);
+    if (!counter) {
+        *grid = (unsigned)(need < 1 ? 1 : need);
+        return cudaSuccess;
+    }
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, smem);
     if (e != cudaSuccess) return e;
     int64_t blocks = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
-    const int64_t need = (n_tiles + (kBlock / 32) - 1) / (kBlock / 32);
     if (blocks > need) blocks = need;
-    if (max_blocks > 0 && blocks > max_blocks) blocks = max_blocks;
     if (blocks < 1) blocks = 1;
     *grid = (unsigned)blocks;
     return cudaSuccess;
@@ -490,7 +510,7 @@ __device__ __forceinline__ bool tile_ray(const RenderParams &p, unsigned long lo
         const int j = ty * kTileH + (slot / kTileW);
         if (i >= p.W || j >= p.H) return false;
         ray = (cam * p.H + j) * p.W + i;
-        const pot_camera *c = p.cams + cam;
+        const pot_camera *c = p.cams ? p.cams + cam : p.few_cams + cam;
         // a1: pixel ray, each operation rounded once in the stated order
         const float xc = __fdiv_rn(__fsub_rn(__fadd_rn((float)i, 0.5f), c->cx), c->fx);
         const float yc = -__fdiv_rn(__fsub_rn(__fadd_rn((float)j, 0.5f), c->cy), c->fy);
@@ -527,17 +547,14 @@ __device__ __forceinline__ void store_ray(const RenderParams &p, int64_t ray, co
 // Forward render, one tile per warp at a time: the warp takes the next tile
 // once all 32 of its rays are done.
 template <int K, typename T, Lookup LOOKUP, bool CAMS, bool COUNT>
-__global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) render_kernel(const RenderParams p)
+__global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) render_kernel(const __grid_constant__ RenderParams p)
 {
     POT_WALK_SHARED(K)
     const int lane = threadIdx.x & 31;
     const T *sig_arr = static_cast<const T *>(p.sigma);
     const T *sh_arr = static_cast<const T *>(p.sh);
-    for (;;) {
-        unsigned long long tile = 0;
-        if (lane == 0) tile = atomicAdd(p.tile_counter, 1ull);
-        tile = __shfl_sync(0xffffffffu, tile, 0);
-        if (tile >= (unsigned long long)p.n_tiles) break;
+    int taken = 0;
+    for (unsigned long long tile; next_tile(p, lane, taken, tile);) {
         float o[3], d[3], near, far;
         int64_t ray;
         const bool has = tile_ray<CAMS>(p, tile, lane, o, d, near, far, ray);
@@ -548,8 +565,7 @@ __global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) render_kern
 }
 
 template <typename T>
-cudaError_t launch_render_t(const RenderParams &p, int K, bool cams, bool count, cudaStream_t s,
-                            int max_blocks)
+cudaError_t launch_render_t(const RenderParams &p, int K, bool cams, bool count, cudaStream_t s)
 {
     using Fn = void (*)(const RenderParams);
     Fn fn = nullptr;
@@ -573,7 +589,7 @@ cudaError_t launch_render_t(const RenderParams &p, int K, bool cams, bool count,
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = walk_smem_bytes(p.cells == nullptr);
     unsigned grid = 0;
-    cudaError_t e = persistent_grid(fn, smem, p.n_tiles, max_blocks, &grid);
+    cudaError_t e = persistent_grid(fn, smem, p.n_tiles, p.tile_counter, &grid);
     if (e != cudaSuccess) return e;
     RenderParams q = p;
     if (cams) set_tile_divs(q);
