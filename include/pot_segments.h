@@ -78,8 +78,8 @@ pot_status pot_render_rays_record(const pot_tree *tree, int64_t n, const float *
  * memory.  Launches on `stream`: the sort of the records by leaf (count,
  * scan, scatter), the per-record kernel, then the walking backward; each
  * reads seg_state on the GPU and returns at once when the other one applies.
- * Scratch from the library's pool: 4 bytes per record slot plus about 12
- * bytes per leaf of the tree.  Float atomics make the summation order, and
+ * Scratch from the library's pool: 12 bytes per record slot plus 4 bytes per
+ * leaf of the tree.  Float atomics make the summation order, and
  * so the last bits of the gradients, vary from call to call (as in
  * pot_render_backward).                                                      */
 pot_status pot_render_backward_recorded(const pot_tree *tree, int64_t n, const float *origins, const float *dirs,

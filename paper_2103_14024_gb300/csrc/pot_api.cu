@@ -1168,8 +1168,6 @@ pot_status pot_render_backward_recorded(const pot_tree *t, int64_t n, const floa
     POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles) ? 0 : 1, true, s), "scratch");
     const SegmentBuffer sb{static_cast<float4 *>(const_cast<void *>(records)), capacity,
                            reinterpret_cast<unsigned long long *>(const_cast<int64_t *>(seg_state))};
-    // scratch of the bin order: bins of 2^bb leaves (count, start, cursor)
-    // and the records' numbers in bin order
     // POT_SEGBWD_ORDER (read once): 1 (default) visits the records in leaf
     // order, 0 in slot order (no sort; as fast when a batch's rays are
     // already neighbours, e.g. whole pixel tiles)
@@ -1177,17 +1175,18 @@ pot_status pot_render_backward_recorded(const pot_tree *t, int64_t n, const floa
         const char *e = std::getenv("POT_SEGBWD_ORDER");
         return e && std::atoi(e) == 0;
     }();
-    // scratch of the leaf order: count, start, cursor per leaf, the scan's
-    // tile sums and the records' numbers in leaf order
+    // scratch of the leaf order: per record its place and its number in leaf order, per leaf its range
     const int64_t nl = t->n_leaves;
-    const int64_t n_tiles = (nl + kSegScanTile - 1) / kSegScanTile;
     Tmp bin_mem;
     SegmentBins bins{};
     if (!direct) {
-        POT_CUDA(bin_mem.alloc(sizeof(unsigned) * (size_t)(3 * nl + 1 + n_tiles + capacity), s), "alloc sort");
-        unsigned *base = static_cast<unsigned *>(bin_mem.p);
-        bins = SegmentBins{base, base + nl, base + 2 * nl + 1, base + 3 * nl + 1 + n_tiles, base + 3 * nl + 1, nl};
-        POT_CUDA(cudaMemsetAsync(bins.count, 0, sizeof(unsigned) * (size_t)nl, s), "clear counts");
+        const size_t n_place = sizeof(uint2) * (size_t)capacity, n_perm = sizeof(unsigned) * (size_t)capacity;
+        POT_CUDA(bin_mem.alloc(n_place + n_perm + sizeof(unsigned) * (size_t)(nl + 1), s), "alloc sort");
+        char *base = static_cast<char *>(bin_mem.p);
+        unsigned *start = reinterpret_cast<unsigned *>(base + n_place + n_perm);
+        bins = SegmentBins{start, start + nl, reinterpret_cast<uint2 *>(base),
+                           reinterpret_cast<unsigned *>(base + n_place), nl};
+        POT_CUDA(cudaMemsetAsync(start, 0, sizeof(unsigned) * (size_t)(nl + 1), s), "clear counts");
     }
     POT_CUDA(launch_backward_recorded(p, t->n_leaves, sb, direct ? nullptr : &bins, grad_rgb, rgb_fwd, grad_sigma,
                                       grad_sh, t->desc.leaf_dtype, t->K, s),

@@ -303,25 +303,38 @@ struct SegBackwardParams {
 #define POT_SEGBWD_MIN_BLOCKS 3
 #endif
 
-// The sum of v over the lanes of each run of adjacent lanes (run0: this
-// lane's run starts there), complete in the run's last lane (a scan within
-// runs).
-__device__ __forceinline__ float run_sum(float v, int lane, int run0)
-{
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const float t = __shfl_up_sync(0xffffffffu, v, d);
-        if (lane - d >= run0) v += t;
-    }
-    return v;
-}
+// How a warp sums 32 records into gradient rows: groups of kLanes lanes, each
+// lane holding kVec adjacent values of a row (kPer times, kLanes * kVec apart),
+// each group taking kRecs consecutive records.
+template <int K>
+struct RowShape {
+    static constexpr int kVec = (3 * K) % 4 == 0 ? 4 : 1;
+    static constexpr int kLanes = 3 * K / kVec < 32 ? 3 * K / kVec : 32;
+    static constexpr int kPer = (3 * K / kVec + kLanes - 1) / kLanes;
+    static constexpr int kGroups = 32 / kLanes;
+    static constexpr int kRecs = (32 + kGroups - 1) / kGroups;
+    // a warp's shared memory, in floats: per record dL/dx as three float4 {x0 x1 x2 x0}, {x1 x2 x0 x1},
+    // {x2 x0 x1 x2} (a lane's four values start with channel 4 l mod 3), the basis (an odd row length keeps
+    // the rows of 32 lanes, and of two groups, on distinct banks), and the leaves
+    static constexpr int kBasisRow = K | 1;
+    static constexpr int kBasis = 32 * 12, kLeaf = kBasis + 32 * kBasisRow, kFloats = (kLeaf + 32 + 3) / 4 * 4;
+};
 
-// Whole warps step over the records together.  Lanes next to each other
-// that hold records of the same leaf (records in leaf order, or neighbouring
-// rays of one forward step in slot order) form a run: the run's terms are
-// summed with shuffles and its last lane issues the float reductions, so a
-// leaf's row gets one set of reductions per warp and step instead of one per
-// record.
+// Whole warps step over the records together, one record per lane.  Lanes next
+// to each other that hold records of the same leaf (records in leaf order, or
+// neighbouring rays of one forward step in slot order) form a run.  A record's
+// row is the product of its three colour derivatives and its basis, so the
+// warp leaves both in shared memory and sums rows from there: a group of lanes
+// holds a whole row (12 lanes x 4 values at K = 16), walks its share of the
+// records and, at the end of a run, adds the row with one reduction instruction
+// of adjacent lanes.
+//
+// What bounds it: the float reductions and the gather of each record's ray and
+// leaf.  One reduction of adjacent 16-byte vectors per row moves whole sectors;
+// it replaced 12 reductions per run of one lane each (a scan of the 49 values
+// over the run by shuffles, 735 instructions a warp), whose 16 bytes each were a
+// request of their own.  With the sort's passes, 2^18 rays on the depth-9 tree
+// (4.2 M records, degree 3): 537 -> 391 us.
 template <int K, typename T>
 __global__ void __launch_bounds__(kFlatBlock, POT_SEGBWD_MIN_BLOCKS) segment_backward_kernel(const SegBackwardParams q)
 {
@@ -332,6 +345,10 @@ __global__ void __launch_bounds__(kFlatBlock, POT_SEGBWD_MIN_BLOCKS) segment_bac
     const int lane = threadIdx.x & 31;
     const T *sig_arr = static_cast<const T *>(q.sigma);
     const T *sh_arr = static_cast<const T *>(q.sh);
+    using S = RowShape<K>;
+    __shared__ float4 rows_sh[kFlatBlock / 32 * S::kFloats / 4];
+    float *ws = reinterpret_cast<float *>(rows_sh) + (threadIdx.x >> 5) * S::kFloats;  // this warp's part
+    const int group = lane / S::kLanes, in_row = lane % S::kLanes;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t k0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); k0 < used; k0 += stride) {
         const int64_t k = k0 + lane;
@@ -366,44 +383,78 @@ __global__ void __launch_bounds__(kFlatBlock, POT_SEGBWD_MIN_BLOCKS) segment_bac
                 }
             }
         }
-        const int prev = __shfl_up_sync(0xffffffffu, leaf, 1);
-        const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || leaf != prev);
-        float *row = q.grad_sh + (int64_t)(leaf < 0 ? 0 : leaf) * (3 * K);
-        if (heads == 0xffffffffu) {  // no two adjacent lanes share a leaf: reductions per lane
-            if (leaf >= 0) {
-                if ((3 * K) % 4 == 0) {
-#pragma unroll
-                    for (int j = 0; j < 3 * K; j += 4)
-                        red_add4(row + j, gx[j % 3] * Y[j / 3], gx[(j + 1) % 3] * Y[(j + 1) / 3],
-                                 gx[(j + 2) % 3] * Y[(j + 2) / 3], gx[(j + 3) % 3] * Y[(j + 3) / 3]);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 3 * K; ++j) red_add(row + j, gx[j % 3] * Y[j / 3]);
-                }
-                if (gsd != 0.f) red_add(q.grad_sigma + leaf, gsd);
-            }
-            continue;
-        }
-        const int run0 = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));  // last head at or before this lane
-        const bool tail = leaf >= 0 && (lane == 31 || ((heads >> (lane + 1)) & 1u));
-        if ((3 * K) % 4 == 0) {
-#pragma unroll
-            for (int j = 0; j < 3 * K; j += 4) {
-                const float v0 = run_sum(gx[j % 3] * Y[j / 3], lane, run0);
-                const float v1 = run_sum(gx[(j + 1) % 3] * Y[(j + 1) / 3], lane, run0);
-                const float v2 = run_sum(gx[(j + 2) % 3] * Y[(j + 2) / 3], lane, run0);
-                const float v3 = run_sum(gx[(j + 3) % 3] * Y[(j + 3) / 3], lane, run0);
-                if (tail) red_add4(row + j, v0, v1, v2, v3);
-            }
+        const int next = __shfl_down_sync(0xffffffffu, leaf, 1);
+        const unsigned ends = __ballot_sync(0xffffffffu, lane == 31 || leaf != next);  // last records of runs
+        if (__all_sync(0xffffffffu, leaf < 0)) continue;
+        if (S::kVec == 4) {
+            float4 *x = reinterpret_cast<float4 *>(ws) + 3 * lane;
+            x[0] = make_float4(gx[0], gx[1], gx[2], gx[0]);
+            x[1] = make_float4(gx[1], gx[2], gx[0], gx[1]);
+            x[2] = make_float4(gx[2], gx[0], gx[1], gx[2]);
         } else {
 #pragma unroll
-            for (int j = 0; j < 3 * K; ++j) {
-                const float v = run_sum(gx[j % 3] * Y[j / 3], lane, run0);
-                if (tail) red_add(row + j, v);
+            for (int c = 0; c < 3; ++c) ws[3 * lane + c] = gx[c];
+        }
+#pragma unroll
+        for (int j = 0; j < K; ++j) ws[S::kBasis + lane * S::kBasisRow + j] = Y.v[j];
+        reinterpret_cast<int *>(ws)[S::kLeaf + lane] = leaf;
+        __syncwarp();
+        if (group < S::kGroups) {
+            float acc[S::kPer][S::kVec];
+#pragma unroll
+            for (int u = 0; u < S::kPer; ++u)
+#pragma unroll
+                for (int v = 0; v < S::kVec; ++v) acc[u][v] = 0.f;
+            const int r_end = min(32, (group + 1) * S::kRecs);
+            for (int r = group * S::kRecs; r < r_end; ++r) {
+                const float *y = ws + S::kBasis + r * S::kBasisRow;
+                if (S::kVec == 4) {
+                    const float4 x = reinterpret_cast<const float4 *>(ws)[3 * r + in_row % 3];
+                    const float y0 = y[4 * in_row / 3], y1 = y[4 * in_row / 3 + 1];
+                    acc[0][0] = fmaf(x.x, y0, acc[0][0]);
+                    acc[0][1 % S::kVec] = fmaf(x.y, in_row % 3 == 2 ? y1 : y0, acc[0][1 % S::kVec]);
+                    acc[0][2 % S::kVec] = fmaf(x.z, in_row % 3 == 0 ? y0 : y1, acc[0][2 % S::kVec]);
+                    acc[0][3 % S::kVec] = fmaf(x.w, y1, acc[0][3 % S::kVec]);
+                } else {
+#pragma unroll
+                    for (int u = 0; u < S::kPer; ++u) {
+                        const int j = u * S::kLanes + in_row;
+                        if (j < 3 * K) acc[u][0] = fmaf(ws[3 * r + j % 3], y[j / 3], acc[u][0]);
+                    }
+                }
+                if (((ends >> r) & 1u) || r + 1 == r_end) {
+                    const int lf = reinterpret_cast<const int *>(ws)[S::kLeaf + r];
+                    if (lf >= 0) {
+                        float *row = q.grad_sh + (int64_t)lf * (3 * K);
+                        if (S::kVec == 4) {
+                            red_add4(row + 4 * in_row, acc[0][0], acc[0][1 % S::kVec], acc[0][2 % S::kVec],
+                                     acc[0][3 % S::kVec]);
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < S::kPer; ++u) {
+                                const int j = u * S::kLanes + in_row;
+                                if (j < 3 * K) red_add(row + j, acc[u][0]);
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < S::kPer; ++u)
+#pragma unroll
+                        for (int v = 0; v < S::kVec; ++v) acc[u][v] = 0.f;
+                }
             }
         }
-        const float gs = run_sum(gsd, lane, run0);
-        if (tail && gs != 0.f) red_add(q.grad_sigma + leaf, gs);
+        // the density derivative: summed over the run by shuffles, complete in its last lane
+        const unsigned before = ends & ((1u << lane) - 1u);
+        const int run0 = before ? 32 - __clz(before) : 0;
+        float gs = gsd;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const float v = __shfl_up_sync(0xffffffffu, gs, d);
+            if (lane - d >= run0) gs += v;
+        }
+        if (leaf >= 0 && ((ends >> lane) & 1u) && gs != 0.f) red_add(q.grad_sigma + leaf, gs);
+        __syncwarp();  // the next records overwrite the rows
     }
 }
 
@@ -431,25 +482,22 @@ cudaError_t launch_segment_backward_t(const SegBackwardParams &q, int K, cudaStr
 }
 
 // ---- recorded segments in leaf order ----------------------------------------
-// The records are visited sorted by leaf (a counting sort: records per leaf,
-// a scan, the record numbers scattered to their leaf's range): a leaf's
-// records are then adjacent, so the per-record kernel merges them within a
-// warp, and neighbouring threads reduce into neighbouring gradient rows.
+// The records are visited leaf by leaf: one pass counts the records per leaf
+// and notes each record's leaf and place among its leaf's, a scan gives every
+// leaf a range of positions, and a second pass puts the record numbers there
+// (without atomics).  A leaf's records are then adjacent, so the per-record
+// kernel merges them within a warp, and neighbouring threads reduce into
+// neighbouring gradient rows.  The leaves' ranges need no particular order: the
+// scan runs over tiles of leaves, each of which draws its range from a counter.
 
 struct SegBinParams {
     SegBackwardParams s;
-    const unsigned *start;  // [n_bins + 1] first sorted position of each leaf
-    unsigned *count;        // [n_bins] records per leaf
-    unsigned *cursor;       // [n_bins] scatter cursors
-    unsigned *perm;         // [capacity] record numbers in leaf order
-    unsigned *tile_sum;     // [ceil(n_bins / kScanTile)] scan partials
-    int64_t n_bins;         // = n_leaves
+    SegmentBins b;
 };
 
 constexpr int kScanBlock = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanTile = kScanBlock * kScanItems;  // counts per scan block
-static_assert(kScanTile == kSegScanTile, "scan tile of the scratch layout");
 
 // A record's leaf, or -1 for an unused slot or one naming an out-of-range ray
 // or leaf.
@@ -468,12 +516,10 @@ __device__ __forceinline__ int64_t records_used(const SegmentBuffer &sb)
     return handed < (unsigned long long)sb.capacity ? (int64_t)handed : sb.capacity;
 }
 
-// Pass 1 (SCATTER = false): records per leaf.  Pass 2 (SCATTER = true): each
-// record's number to its leaf's range of perm.  Whole warps step together so
-// that lanes with the same leaf (neighbouring rays of one step) share one
-// atomic, found with a match.
-template <bool SCATTER>
-__global__ void __launch_bounds__(kFlatBlock) leaf_pass_kernel(const SegBinParams q)
+// Pass 1: records per leaf, and each record's leaf and place.  Whole warps step
+// together so that lanes with the same leaf (neighbouring rays of one step)
+// share one atomic, found with a match.
+__global__ void __launch_bounds__(kFlatBlock) leaf_count_kernel(const SegBinParams q)
 {
     if (q.s.sb.state[1] != 0ull) return;
     const int64_t used = records_used(q.s.sb);
@@ -481,17 +527,24 @@ __global__ void __launch_bounds__(kFlatBlock) leaf_pass_kernel(const SegBinParam
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); i0 < used; i0 += stride) {
         const int64_t i = i0 + lane;
-        const int b = record_leaf(q.s, i, used);
-        const unsigned m = __match_any_sync(0xffffffffu, b);
+        const int leaf = record_leaf(q.s, i, used);
+        const unsigned m = __match_any_sync(0xffffffffu, leaf);
         const int leader = __ffs(m) - 1;
-        if (!SCATTER) {
-            if (b >= 0 && lane == leader) atomicAdd(q.count + b, (unsigned)__popc(m));
-        } else {
-            unsigned base = 0;
-            if (b >= 0 && lane == leader) base = atomicAdd(q.cursor + b, (unsigned)__popc(m));
-            base = __shfl_sync(m, base, leader);
-            if (b >= 0) q.perm[q.start[b] + base + __popc(m & ((1u << lane) - 1u))] = (unsigned)i;
-        }
+        unsigned base = 0;
+        if (leaf >= 0 && lane == leader) base = atomicAdd(q.b.start + leaf, (unsigned)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, leader);
+        if (i < used) q.b.place[i] = make_uint2((unsigned)leaf, base + __popc(m & ((1u << lane) - 1u)));
+    }
+}
+
+// Pass 2: each record's number to its position.
+__global__ void __launch_bounds__(kFlatBlock) leaf_scatter_kernel(const SegBinParams q)
+{
+    if (q.s.sb.state[1] != 0ull) return;
+    const int64_t used = records_used(q.s.sb);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < used; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint2 v = q.b.place[i];
+        if ((int)v.x >= 0) q.b.perm[q.b.start[v.x] + v.y] = (unsigned)i;
     }
 }
 
@@ -523,56 +576,27 @@ __device__ __forceinline__ unsigned block_exclusive_scan(unsigned v, unsigned *t
     return (wid ? warp_sum[wid - 1] : 0u) + incl - v;
 }
 
-// Scan step 1: the sum of each tile of kScanTile counts.
-__global__ void __launch_bounds__(kScanBlock) scan_tile_sums_kernel(const SegBinParams q)
+// Counts become first positions, a tile of kScanTile leaves per block.
+__global__ void __launch_bounds__(kScanBlock) leaf_ranges_kernel(const SegBinParams q)
 {
-    const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-    unsigned v = 0;
-#pragma unroll
-    for (int u = 0; u < kScanItems; ++u)
-        if (base + u < q.n_bins) v += q.count[base + u];
-    unsigned total;
-    block_exclusive_scan(v, &total);
-    if (threadIdx.x == 0) q.tile_sum[blockIdx.x] = total;
-}
-
-// Scan step 2 (one block): the tile sums become the tiles' exclusive offsets;
-// start[n_bins] = the number of records.
-__global__ void __launch_bounds__(kScanBlock) scan_tile_offsets_kernel(const SegBinParams q, int64_t n_tiles)
-{
-    const int64_t per = (n_tiles + kScanBlock - 1) / kScanBlock;
-    const int64_t lo = threadIdx.x * per, hi = min(lo + per, n_tiles);
-    unsigned v = 0;
-    for (int64_t t = lo; t < hi; ++t) v += q.tile_sum[t];
-    unsigned total;
-    unsigned run = block_exclusive_scan(v, &total);
-    for (int64_t t = lo; t < hi; ++t) {
-        const unsigned c = q.tile_sum[t];
-        q.tile_sum[t] = run;
-        run += c;
-    }
-    if (threadIdx.x == 0) const_cast<unsigned *>(q.start)[q.n_bins] = total;
-}
-
-// Scan step 3: each leaf's first sorted position; cursors cleared.
-__global__ void __launch_bounds__(kScanBlock) scan_apply_kernel(const SegBinParams q)
-{
+    __shared__ unsigned tile_base;
+    if (q.s.sb.state[1] != 0ull) return;
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
     unsigned c[kScanItems], v = 0;
 #pragma unroll
     for (int u = 0; u < kScanItems; ++u) {
-        c[u] = base + u < q.n_bins ? q.count[base + u] : 0u;
+        c[u] = base + u < q.b.n_bins ? q.b.start[base + u] : 0u;
         v += c[u];
     }
     unsigned total;
-    unsigned run = block_exclusive_scan(v, &total) + q.tile_sum[blockIdx.x];
-    unsigned *start = const_cast<unsigned *>(q.start);
+    unsigned run = block_exclusive_scan(v, &total);
+    if (threadIdx.x == 0) tile_base = total ? atomicAdd(q.b.n_perm, total) : 0u;
+    __syncthreads();
+    if (total == 0) return;
+    run += tile_base;
 #pragma unroll
     for (int u = 0; u < kScanItems; ++u) {
-        if (base + u < q.n_bins) {
-            start[base + u] = run;
-            q.cursor[base + u] = 0u;
-        }
+        if (base + u < q.b.n_bins) q.b.start[base + u] = run;
         run += c[u];
     }
 }
@@ -588,17 +612,15 @@ cudaError_t launch_leaf_order_t(const SegBinParams &q, int K, cudaStream_t s)
     int64_t blocks = (q.s.sb.capacity + kFlatBlock - 1) / kFlatBlock;
     if (blocks > 8 * (int64_t)sms) blocks = 8 * (int64_t)sms;
     if (blocks < 1) blocks = 1;
-    const int64_t n_tiles = (q.n_bins + kScanTile - 1) / kScanTile;
-    leaf_pass_kernel<false><<<(unsigned)blocks, kFlatBlock, 0, s>>>(q);
-    scan_tile_sums_kernel<<<(unsigned)n_tiles, kScanBlock, 0, s>>>(q);
-    scan_tile_offsets_kernel<<<1, kScanBlock, 0, s>>>(q, n_tiles);
-    scan_apply_kernel<<<(unsigned)n_tiles, kScanBlock, 0, s>>>(q);
-    leaf_pass_kernel<true><<<(unsigned)blocks, kFlatBlock, 0, s>>>(q);
-    count_launch(5);
+    const int64_t n_tiles = (q.b.n_bins + kScanTile - 1) / kScanTile;
+    leaf_count_kernel<<<(unsigned)blocks, kFlatBlock, 0, s>>>(q);
+    leaf_ranges_kernel<<<(unsigned)n_tiles, kScanBlock, 0, s>>>(q);
+    leaf_scatter_kernel<<<(unsigned)blocks, kFlatBlock, 0, s>>>(q);
+    count_launch(3);
     // the per-record kernel over the records in leaf order
     SegBackwardParams sq = q.s;
-    sq.perm = q.perm;
-    sq.n_perm = q.start + q.n_bins;
+    sq.perm = q.b.perm;
+    sq.n_perm = q.b.n_perm;
     return launch_segment_backward_t<T>(sq, K, s);
 }
 
@@ -814,7 +836,7 @@ cudaError_t launch_backward_recorded(const RenderParams &r, int64_t n_leaves, co
                         r.sh,    r.ray_d,    grad_rgb, rgb_fwd,    grad_sigma, grad_sh};
     cudaError_t e;
     if (bins) {
-        const SegBinParams bq{q, bins->start, bins->count, bins->cursor, bins->perm, bins->tile_sum, bins->n_bins};
+        const SegBinParams bq{q, *bins};
         switch (dtype) {
         case POT_F32: e = launch_leaf_order_t<float>(bq, K, s); break;
         case POT_F16: e = launch_leaf_order_t<__half>(bq, K, s); break;

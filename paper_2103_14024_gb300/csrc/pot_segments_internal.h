@@ -21,15 +21,13 @@ struct SegmentBuffer {
 cudaError_t launch_render_record(const RenderParams &p, const SegmentBuffer &sb, int dtype, int K, cudaStream_t s);
 
 // Scratch of the per-record backward in leaf order (a counting sort of the
-// records by leaf); count zeroed by the caller.
-constexpr int kSegScanTile = 4096;  // counts per block of the scan
+// records by leaf); start and n_perm zeroed by the caller.
 struct SegmentBins {
-    unsigned *count;     // [n_bins]
-    unsigned *start;     // [n_bins + 1]
-    unsigned *cursor;    // [n_bins]
-    unsigned *perm;      // [capacity]
-    unsigned *tile_sum;  // [ceil(n_bins / kSegScanTile)]
-    int64_t n_bins;      // = the tree's leaves
+    unsigned *start;   // [n_bins] records per leaf, then the leaf's first position
+    unsigned *n_perm;  // [1] positions handed out
+    uint2 *place;      // [capacity] each record's leaf and place among its leaf's records
+    unsigned *perm;    // [capacity] record numbers by position
+    int64_t n_bins;    // = the tree's leaves
 };
 
 // Gradients from the records, one thread per record with float reductions,
