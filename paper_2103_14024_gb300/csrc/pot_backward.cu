@@ -168,8 +168,10 @@ struct BackwardParams {
 enum BackwardMode { kGradAndColour = 0, kGrad = 1, kMseTarget = 2 };
 
 #ifndef POT_BACKWARD_MIN_BLOCKS
-// resident blocks per SM: 4 (16 warps, at most 128 registers)
-#define POT_BACKWARD_MIN_BLOCKS 4
+// resident blocks per SM: 3 (12 warps, 168 registers).  4 blocks: 692 against
+// 702 us on 2^18 random pixels of the depth-9 tree, but 2928 against 2649 us where
+// every ray meets a leaf (see rays_min_blocks); 5: 814 us; 6: 908 us
+#define POT_BACKWARD_MIN_BLOCKS 3
 #endif
 
 // MODE kGradAndColour: dL/dC and C given; kGrad: dL/dC given, C from a first

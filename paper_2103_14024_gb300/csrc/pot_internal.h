@@ -168,7 +168,8 @@ cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_
 
 // Whether n_tiles tiles are all resident at once in every walk kernel (16 warps
 // per SM at least): then warp i takes tile i, and the launch needs no tile
-// counter, that is no allocation and no memset before it.
+// counter, that is no allocation and no memset before it.  (With the cameras in
+// the launch too, one 256 x 256 view 88 -> 77 us, one 64 x 64 view 26 -> 23 us.)
 bool one_wave(int64_t n_tiles);
 
 // cameras interleaved per tile group in camera renders (POT_VIEW_GROUP overrides)

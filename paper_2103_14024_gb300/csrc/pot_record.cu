@@ -13,10 +13,6 @@
 #include "pot_render.cuh"
 #include "pot_segments_internal.h"
 
-#ifndef POT_RECORD_MIN_BLOCKS
-#define POT_RECORD_MIN_BLOCKS 6  // resident blocks per SM: 80 registers, no spills
-#endif
-
 namespace pot {
 
 namespace {
@@ -43,7 +39,7 @@ struct RecordVisitor {
 };
 
 template <int K, typename T, Lookup LOOKUP>
-__global__ void __launch_bounds__(kBlock, POT_RECORD_MIN_BLOCKS)
+__global__ void __launch_bounds__(kBlock, rays_min_blocks(LOOKUP))
     record_kernel(const __grid_constant__ RenderParams p, const SegmentBuffer sb)
 {
     POT_WALK_SHARED(K)

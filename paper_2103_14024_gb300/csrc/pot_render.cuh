@@ -38,11 +38,20 @@ enum Lookup { kLookDense, kLookBrick, kLookAny };
 // against 7.32 ms).  72 registers (28 warps): 89 us, 340 us, 5.65 ms, 7.33 ms.
 // With bricks a step waits for two loads in turn, and 32 warps are better (one
 // full-HD view at depth 10: 768 against 801 us).
+// Explicit rays need not have neighbours in their warp, and then every lane
+// brings its own lines: fewer resident warps keep more of them in L1.  4 blocks
+// against 6, 2^18 random pixels of 100 views on the depth-9 tree (one in four
+// meets a leaf): render_rays 368 against 400 us, where every ray meets a leaf
+// 725 against 934 us; the recording forward 440 against 494 and 860 against
+// 1118 us (3 and 2 blocks the same within 1 %, as their registers allow 4).
+// The descent of the child array, a chain of loads, wants 24 warps there (no
+// index, 2^18 random pixels: 736 against 805 us).
 constexpr int kBlock = 128;
 #ifndef POT_RENDER_MIN_BLOCKS
 #define POT_RENDER_MIN_BLOCKS 6
 #endif
-constexpr int render_min_blocks(Lookup l) { return l == kLookDense ? POT_RENDER_MIN_BLOCKS : 8; }
+constexpr int render_min_blocks(Lookup l) { return l == kLookBrick ? 8 : POT_RENDER_MIN_BLOCKS; }
+constexpr int rays_min_blocks(Lookup l) { return l == kLookAny ? 6 : 4; }  // explicit rays
 
 // Fixed-point ray times.  A walk measures time from the clip range's entry
 // tin in units of 2^-kTimeFrac, with the ray's direction scaled by a power of
@@ -547,7 +556,8 @@ __device__ __forceinline__ void store_ray(const RenderParams &p, int64_t ray, co
 // Forward render, one tile per warp at a time: the warp takes the next tile
 // once all 32 of its rays are done.
 template <int K, typename T, Lookup LOOKUP, bool CAMS, bool COUNT>
-__global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) render_kernel(const __grid_constant__ RenderParams p)
+__global__ void __launch_bounds__(kBlock, CAMS ? render_min_blocks(LOOKUP) : rays_min_blocks(LOOKUP))
+    render_kernel(const __grid_constant__ RenderParams p)
 {
     POT_WALK_SHARED(K)
     const int lane = threadIdx.x & 31;
