@@ -53,7 +53,7 @@ WalkFrame walk_frame(float size, int depth)
     return f;
 }
 
-bool one_wave(int64_t n_tiles)
+bool one_wave(int64_t n_tiles, int *part_log2)
 {
     static std::atomic<int> sms[64];
     int dev = 0;
@@ -63,7 +63,11 @@ bool one_wave(int64_t n_tiles)
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
         sms[dev].store(n, std::memory_order_relaxed);
     }
-    return n_tiles <= 16ll * n;
+    if (n_tiles > 16ll * n) return false;
+    int l = 0;
+    while (l < kMaxPartLog2 && (n_tiles << (l + 1)) <= (int64_t)kPartWarps * n) ++l;
+    *part_log2 = l;
+    return true;
 }
 
 int render_view_group(int n_cams)
@@ -810,7 +814,7 @@ pot_status pot_render(const pot_tree *t, const pot_camera *cams, int32_t n_cams,
     const bool host_out = !is_device_ptr(rgb) || (t_final && !is_device_ptr(t_final));
     p.n_tiles = p.tiles_per_cam * n_cams;
     // a host-memory output renders in chunks, one counter each
-    const int n_counters = host_out ? n_cams : one_wave(p.n_tiles) ? 0 : 1;
+    const int n_counters = host_out ? n_cams : one_wave(p.n_tiles, &p.part_log2) ? 0 : 1;
     POT_CUDA(walk_scratch(p, scratch, cams, n_cams, n_counters, !host_out, s), "scratch");
     if (host_out) return render_to_host(p, t, p.cams, n_cams, rgb, t_final, s);
     p.n_cams = n_cams;
@@ -853,7 +857,7 @@ pot_status pot_render_rays(const pot_tree *t, int64_t n, const float *origins, c
     p.n_tiles = (n + 31) / 32;
     p.rgb = (float *)drgb;
     p.t_final = (float *)dtf;
-    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles) ? 0 : 1, true, s), "scratch");
+    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles, &p.part_log2) ? 0 : 1, true, s), "scratch");
     POT_CUDA(launch_render(p, t, false, s), "render_rays");
     POT_CUDA(orgb.finish(s), "copy rgb");
     POT_CUDA(otf.finish(s), "copy t_final");
@@ -893,7 +897,7 @@ pot_status pot_visibility(const pot_tree *t, const pot_camera *cams, int32_t n_c
     if (p.tiles_per_cam * ((int64_t)n_cams + 16) >= (1ll << 32))
         return tile_limit_error();
     p.n_tiles = p.tiles_per_cam * n_cams;
-    POT_CUDA(walk_scratch(p, scratch, cams, n_cams, one_wave(p.n_tiles) ? 0 : 1, true, s), "scratch");
+    POT_CUDA(walk_scratch(p, scratch, cams, n_cams, one_wave(p.n_tiles, &p.part_log2) ? 0 : 1, true, s), "scratch");
     POT_CUDA(launch_visibility(p, t, max_weight, s), "visibility");
     return POT_OK;
 }
@@ -1030,7 +1034,7 @@ pot_status pot_render_backward(const pot_tree *t, int64_t n, const float *origin
     p.near = near;
     p.far = far;
     p.n_tiles = (n + 31) / 32;
-    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles) ? 0 : 1, true, s), "scratch");
+    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles, &p.part_log2) ? 0 : 1, true, s), "scratch");
     POT_CUDA(launch_backward(p, grad_rgb, rgb_fwd, grad_sigma, grad_sh, t->desc.leaf_dtype, t->K, s), "backward");
     return POT_OK;
 }
@@ -1069,7 +1073,7 @@ pot_status pot_render_mse_backward(const pot_tree *t, int64_t n, const float *or
     p.near = near;
     p.far = far;
     p.n_tiles = (n + 31) / 32;
-    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles) ? 0 : 1, true, s), "scratch");
+    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles, &p.part_log2) ? 0 : 1, true, s), "scratch");
     POT_CUDA(launch_mse_backward(p, target, rgb, loss, grad_sigma, grad_sh, t->desc.leaf_dtype, t->K, s),
              "mse backward");
     return POT_OK;
@@ -1125,7 +1129,7 @@ pot_status pot_render_rays_record(const pot_tree *t, int64_t n, const float *ori
     p.n_tiles = (n + 31) / 32;
     p.rgb = rgb;
     p.t_final = t_final;
-    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles) ? 0 : 1, true, s), "scratch");
+    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles, &p.part_log2) ? 0 : 1, true, s), "scratch");
     const SegmentBuffer sb{static_cast<float4 *>(records), capacity, reinterpret_cast<unsigned long long *>(seg_state)};
     POT_CUDA(launch_render_record(p, sb, t->desc.leaf_dtype, t->K, s), "render_rays_record");
     return POT_OK;
@@ -1165,7 +1169,7 @@ pot_status pot_render_backward_recorded(const pot_tree *t, int64_t n, const floa
     p.near = near;
     p.far = far;
     p.n_tiles = (n + 31) / 32;
-    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles) ? 0 : 1, true, s), "scratch");
+    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles, &p.part_log2) ? 0 : 1, true, s), "scratch");
     const SegmentBuffer sb{static_cast<float4 *>(const_cast<void *>(records)), capacity,
                            reinterpret_cast<unsigned long long *>(const_cast<int64_t *>(seg_state))};
     // POT_SEGBWD_ORDER (read once): 1 (default) visits the records in leaf

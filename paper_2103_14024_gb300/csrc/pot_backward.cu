@@ -186,11 +186,11 @@ __global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kern
     const int lane = threadIdx.x & 31;
     const T *sig_arr = static_cast<const T *>(p.sigma);
     const T *sh_arr = static_cast<const T *>(p.sh);
-    int taken = 0;
-    for (unsigned long long tile; next_tile(p, lane, taken, tile);) {
-        const int64_t ray = (int64_t)tile * 32 + lane;
+    int taken = 0, slot;
+    for (unsigned long long tile; next_tile(p, lane, taken, tile, slot);) {
+        const int64_t ray = (int64_t)tile * 32 + slot;
         float lsum = 0.f;  // this ray's squared error (MSE mode)
-        const bool has = ray < p.n_rays;
+        const bool has = slot < 32 && ray < p.n_rays;
         float o[3], d[3];
         GradVisitor<K, T> gv;
         gv.sig_arr = sig_arr;
@@ -254,7 +254,7 @@ cudaError_t launch_backward_t(const BackwardParams &bp, int K, int mode, cudaStr
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = walk_smem_bytes(bp.r.cells == nullptr);
     unsigned grid = 0;
-    cudaError_t e = persistent_grid(fn, smem, bp.r.n_tiles, bp.r.tile_counter, &grid);
+    cudaError_t e = persistent_grid(fn, smem, bp.r, &grid);
     if (e != cudaSuccess) return e;
     fn<<<grid, kBlock, smem, s>>>(bp);
     count_launch();

@@ -35,11 +35,11 @@ __global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) visibility_
     POT_WALK_SHARED(K)
     const int lane = threadIdx.x & 31;
     const T *sig_arr = static_cast<const T *>(p.sigma);
-    int taken = 0;
-    for (unsigned long long tile; next_tile(p, lane, taken, tile);) {
+    int taken = 0, slot;
+    for (unsigned long long tile; next_tile(p, lane, taken, tile, slot);) {
         float o[3], d[3], near, far;
         int64_t ray;
-        const bool has = tile_ray<true>(p, tile, lane, o, d, near, far, ray);
+        const bool has = tile_ray<true>(p, tile, slot, o, d, near, far, ray);
         MaxWeightVisitor<T> v{sig_arr, p.gamma, 1.f, max_w};
         walk_rays<K, T, LOOKUP, true>(p, stk, ysm, wst, has, o, d, near, far, v);
     }
@@ -53,7 +53,7 @@ cudaError_t launch_visibility_t(const RenderParams &p, int K, float *max_w, cuda
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = walk_smem_bytes(p.cells == nullptr);
     unsigned grid = 0;
-    cudaError_t e = persistent_grid(fn, smem, p.n_tiles, p.tile_counter, &grid);
+    cudaError_t e = persistent_grid(fn, smem, p, &grid);
     if (e != cudaSuccess) return e;
     RenderParams q = p;
     set_tile_divs(q);

@@ -110,7 +110,8 @@ struct RenderParams {
     int32_t *seg_count;
     uint8_t *leaf_touched;
     // scratch
-    unsigned long long *tile_counter;  // null: one tile per warp, in order
+    unsigned long long *tile_counter;  // null: the tiles in order, 1 << part_log2 warps to a tile
+    int part_log2;                     // (without a counter) each with 32 >> part_log2 of its rays
     unsigned int *err;
     // cameras of calls with few of them: they travel in the launch instead of
     // a copy of their own ahead of it
@@ -167,10 +168,17 @@ cudaError_t quantize_tree(const pot_tree *t, int bits, pot_tree *q, cudaStream_t
 cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_t s, unsigned int *err);
 
 // Whether n_tiles tiles are all resident at once in every walk kernel (16 warps
-// per SM at least): then warp i takes tile i, and the launch needs no tile
-// counter, that is no allocation and no memset before it.  (With the cameras in
-// the launch too, one 256 x 256 view 88 -> 77 us, one 64 x 64 view 26 -> 23 us.)
-bool one_wave(int64_t n_tiles);
+// per SM at least): then the tiles go to the warps in order, and the launch needs
+// no tile counter, that is no allocation and no memset before it.  (With the
+// cameras in the launch too, one 256 x 256 view 88 -> 77 us, one 64 x 64 view
+// 26 -> 23 us.)  *part_log2: into how many warps a tile is split, as long as
+// kPartWarps per SM are not filled (24: one 200 x 200 f32 view 235 -> 217 us, fused
+// training call of 20,011 rays 92 -> 84 us; 48: 201 and 109 us; 16: 235 and 86 us).
+#ifndef POT_PART_WARPS
+#define POT_PART_WARPS 24
+#endif
+constexpr int kPartWarps = POT_PART_WARPS, kMaxPartLog2 = 4;
+bool one_wave(int64_t n_tiles, int *part_log2);
 
 // cameras interleaved per tile group in camera renders (POT_VIEW_GROUP overrides)
 int render_view_group(int n_cams);

@@ -53,16 +53,17 @@ __global__ void __launch_bounds__(kBlock, rays_min_blocks(LOOKUP))
     long long base = -1;
     int fill = kSegBlock;
     bool dead = false;
-    int taken = 0;
-    for (unsigned long long tile; next_tile(p, lane, taken, tile);) {
-        const int64_t ray = (int64_t)tile * 32 + lane;
+    int taken = 0, part;
+    for (unsigned long long tile; next_tile(p, lane, taken, tile, part);) {
+        const int64_t ray = (int64_t)tile * 32 + part;
+        const bool has = part < 32 && ray < p.n_rays;
         RecordVisitor<K, T> v;
         v.sv = ShadeVisitor<K, T, false>{sig_arr, sh_arr, nullptr, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, nullptr};
         v.has = false;
         Walker<K, T, LOOKUP> w;
         w.ysm = ysm;
         w.st = wst;
-        bool alive = ray < p.n_rays;
+        bool alive = has;
         float o[3], d[3];
         if (alive) {
 #pragma unroll
@@ -109,7 +110,7 @@ __global__ void __launch_bounds__(kBlock, rays_min_blocks(LOOKUP))
                 r[1] = make_float4(v.P0[0], v.P0[1], v.P0[2], 0.f);
             }
         }
-        if (ray < p.n_rays) store_ray<K, T, false>(p, ray, v.sv);
+        if (has) store_ray<K, T, false>(p, ray, v.sv);
     }
     // the slots of the last block that this warp did not use
     if (base >= 0)
@@ -125,7 +126,7 @@ cudaError_t launch_record_t(const RenderParams &p, const SegmentBuffer &sb, int 
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = walk_smem_bytes(p.cells == nullptr);
     unsigned grid = 0;
-    cudaError_t e = persistent_grid(fn, smem, p.n_tiles, p.tile_counter, &grid);
+    cudaError_t e = persistent_grid(fn, smem, p, &grid);
     if (e != cudaSuccess) return e;
     fn<<<grid, kBlock, smem, s>>>(p, sb);
     count_launch();

@@ -392,30 +392,38 @@ inline bool dense_index(const RenderParams &p) { return p.cells && !p.btab; }
 #define POT_PICK_WALK(FN, K, T, DENSE, ...)                                                                     \
     ((DENSE) ? POT_PICK_K(FN, K, T, kLookDense, ##__VA_ARGS__) : POT_PICK_K(FN, K, T, kLookAny, ##__VA_ARGS__))
 
-// The next tile of a warp: from the launch's counter until none is left, or,
-// without one, the tile of the warp's place in the grid, once (taken counts the
-// calls).  False when there is none.
-__device__ __forceinline__ bool next_tile(const RenderParams &p, int lane, int &taken, unsigned long long &tile)
+// The next tile of a warp, and the lane's slot in it (0..31; 32 for a lane that
+// takes none): from the launch's counter until none is left, or, without one,
+// once, by the warp's place in the grid.  Launches with fewer tiles than warps
+// that could be resident split them: the time of such a launch is that of its
+// slowest warp, and with fewer rays a warp takes fewer sides of the branches, waits
+// for fewer lines per load and ends with its own rays.  False when there is none.
+__device__ __forceinline__ bool next_tile(const RenderParams &p, int lane, int &taken, unsigned long long &tile,
+                                          int &slot)
 {
+    slot = lane;
     if (p.tile_counter) {
         tile = 0;
         if (lane == 0) tile = atomicAdd(p.tile_counter, 1ull);
         tile = __shfl_sync(0xffffffffu, tile, 0);
     } else {
         if (taken++) return false;
-        tile = (unsigned long long)blockIdx.x * (kBlock / 32) + (threadIdx.x >> 5);
+        const unsigned warp = blockIdx.x * (kBlock / 32) + (threadIdx.x >> 5);
+        const int rays = 32 >> p.part_log2;
+        tile = warp >> p.part_log2;
+        slot = lane < rays ? (int)(warp & ((1u << p.part_log2) - 1u)) * rays + lane : 32;
     }
     return tile < (unsigned long long)p.n_tiles;
 }
 
-// Grid of a walk kernel: a block per kBlock / 32 tiles where every warp takes one
-// (counter null), else one wave of resident blocks (SMs x blocks
+// Grid of a walk kernel: all warps of all tiles without a counter, else one wave of resident blocks (SMs x blocks
 // per SM for this kernel and shared memory), no more blocks than tiles need.
 template <typename Fn>
-cudaError_t persistent_grid(Fn fn, size_t smem, int64_t n_tiles, const void *counter, unsigned *grid)
+cudaError_t persistent_grid(Fn fn, size_t smem, const RenderParams &p, unsigned *grid)
 {
-    const int64_t need = (n_tiles + (kBlock / 32) - 1) / (kBlock / 32);
-    if (!counter) {
+    const int64_t warps = p.tile_counter ? p.n_tiles : p.n_tiles << p.part_log2;
+    const int64_t need = (warps + (kBlock / 32) - 1) / (kBlock / 32);
+    if (!p.tile_counter) {
         *grid = (unsigned)(need < 1 ? 1 : need);
         return cudaSuccess;
     }
@@ -517,7 +525,7 @@ __device__ __forceinline__ bool tile_ray(const RenderParams &p, unsigned long lo
         const int tx = (int)(rem - (uint32_t)ty * (uint32_t)p.tiles_x);
         const int i = tx * kTileW + (slot % kTileW);
         const int j = ty * kTileH + (slot / kTileW);
-        if (i >= p.W || j >= p.H) return false;
+        if (slot >= 32 || i >= p.W || j >= p.H) return false;
         ray = (cam * p.H + j) * p.W + i;
         const pot_camera *c = p.cams ? p.cams + cam : p.few_cams + cam;
         // a1: pixel ray, each operation rounded once in the stated order
@@ -533,7 +541,7 @@ __device__ __forceinline__ bool tile_ray(const RenderParams &p, unsigned long lo
         return true;
     }
     ray = (int64_t)tile * 32 + slot;
-    if (ray >= p.n_rays) return false;
+    if (slot >= 32 || ray >= p.n_rays) return false;
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
         o[r] = __ldg(p.ray_o + 3 * ray + r);
@@ -563,11 +571,11 @@ __global__ void __launch_bounds__(kBlock, CAMS ? render_min_blocks(LOOKUP) : ray
     const int lane = threadIdx.x & 31;
     const T *sig_arr = static_cast<const T *>(p.sigma);
     const T *sh_arr = static_cast<const T *>(p.sh);
-    int taken = 0;
-    for (unsigned long long tile; next_tile(p, lane, taken, tile);) {
+    int taken = 0, slot;
+    for (unsigned long long tile; next_tile(p, lane, taken, tile, slot);) {
         float o[3], d[3], near, far;
         int64_t ray;
-        const bool has = tile_ray<CAMS>(p, tile, lane, o, d, near, far, ray);
+        const bool has = tile_ray<CAMS>(p, tile, slot, o, d, near, far, ray);
         ShadeVisitor<K, T, COUNT> v{sig_arr, sh_arr, p.leaf_touched, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, p.codebook};
         walk_rays<K, T, LOOKUP, CAMS>(p, stk, ysm, wst, has, o, d, near, far, v);
         if (has) store_ray<K, T, COUNT>(p, ray, v);
@@ -599,7 +607,7 @@ cudaError_t launch_render_t(const RenderParams &p, int K, bool cams, bool count,
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = walk_smem_bytes(p.cells == nullptr);
     unsigned grid = 0;
-    cudaError_t e = persistent_grid(fn, smem, p.n_tiles, p.tile_counter, &grid);
+    cudaError_t e = persistent_grid(fn, smem, p, &grid);
     if (e != cudaSuccess) return e;
     RenderParams q = p;
     if (cams) set_tile_divs(q);
