@@ -629,8 +629,6 @@ cudaError_t launch_leaf_order_t(const SegBinParams &q, int K, cudaStream_t s)
 // ---- optimiser step on the leaves ------------------------------------------
 struct StepParams {
     int64_t L;
-    int K3;      // 3K
-    int stride;  // SH record stride (elements)
     float lr_sigma, lr_sh, alpha, beta1, beta2, eps;
     float bc1, bc2;  // Adam bias corrections 1 - beta^t
 };
@@ -674,77 +672,74 @@ __device__ __forceinline__ void store_state(float *state, int64_t N, int64_t j, 
     }
 }
 
-// FLAT: the SH records have no padding (stride == 3K), so the public
-// gradient index is the record index and no division is needed.
-template <int KIND, bool FLAT>
-__global__ void k_step(StepParams sp, float *sigma, float *sh, const float *gs, const float *gsh, float *state)
+// The step streams L (1 + 3K) values through 3 (SGD) to 7 (Adam) arrays and is
+// bound by HBM.  Work goes in units of kStepUnit values, first the densities,
+// then the SH values in the gradients' order; a thread takes every kStepBlock-th
+// value of a unit and has the loads of all of them in flight before the first
+// update.  Accesses are 4 bytes and adjacent across a warp, as the state's SH part
+// starts at an offset of L floats, which no vector access can count on.  (One
+// value per thread and iteration moved 4.6 TB/s, or 6.7 TB/s with 16-byte vectors
+// where the leaves were a multiple of 4: the RMSprop step of 4,026,531 leaves at
+// degree 3 860 -> 556 us = 7.1 TB/s, of 4,026,528 leaves 587 -> 551 us, of 4.0 M
+// leaves at degree 2, whose records are padded, 541 -> 442 us.)
+constexpr int kStepBlock = 256, kStepPer = 8, kStepUnit = kStepBlock * kStepPer;
+
+template <int KIND, int K>
+__global__ void __launch_bounds__(kStepBlock) k_step(StepParams sp, float *__restrict__ sigma, float *__restrict__ sh,
+                                                     const float *__restrict__ gs, const float *__restrict__ gsh,
+                                                     float *__restrict__ state)
 {
-    const int64_t N = sp.L * (1 + sp.K3);
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x) {
-        float *param;
-        float g, lr;
-        if (j < sp.L) {
-            param = sigma + j;
-            g = gs[j];
-            lr = sp.lr_sigma;
-        } else {
-            const int64_t jj = j - sp.L;
-            if (FLAT) {
-                param = sh + jj;
-            } else {
-                const int64_t i = jj / sp.K3;
-                param = sh + i * sp.stride + (jj - i * sp.K3);
+    constexpr int K3 = 3 * K, STRIDE = sh_stride<float>(K);
+    const int64_t N = sp.L * (1 + K3);
+    const int64_t sig_units = (sp.L + kStepUnit - 1) / kStepUnit;
+    const int64_t units = sig_units + (sp.L * K3 + kStepUnit - 1) / kStepUnit;
+    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+        const bool dens = u < sig_units;
+        const int64_t base = (dens ? u : u - sig_units) * kStepUnit, end = dens ? sp.L : sp.L * K3;
+        const int64_t row0 = base / K3;
+        const int rem = (int)(base - row0 * K3);
+        const float *grad = dens ? gs : gsh;
+        float *param = dens ? sigma : sh, *st = dens ? state : state + sp.L;
+        const float lr = dens ? sp.lr_sigma : sp.lr_sh;
+        float x[kStepPer], g[kStepPer], m[kStepPer], v[kStepPer];
+        // a value's place in the padded records: its row and column, by 32-bit division by a constant
+        auto at = [&](int i) -> int64_t {
+            const int e = i * kStepBlock + (int)threadIdx.x;
+            if (dens || STRIDE == K3) return base + e;
+            const unsigned r = (unsigned)(rem + e) / (unsigned)K3;
+            return (row0 + r) * STRIDE + ((unsigned)(rem + e) - r * (unsigned)K3);
+        };
+#pragma unroll
+        for (int i = 0; i < kStepPer; ++i) {
+            const int64_t j = base + i * kStepBlock + threadIdx.x;
+            m[i] = v[i] = x[i] = g[i] = 0.f;
+            if (j < end) {
+                x[i] = param[at(i)];
+                g[i] = grad[j];
+                load_state<KIND>(st, N, j, m[i], v[i]);
             }
-            g = gsh[jj];
-            lr = sp.lr_sh;
         }
-        float m = 0.f, v = 0.f;
-        load_state<KIND>(state, N, j, m, v);
-        *param = step_one<KIND>(sp, *param, g, lr, m, v);
-        store_state<KIND>(state, N, j, m, v);
+#pragma unroll
+        for (int i = 0; i < kStepPer; ++i) {
+            const int64_t j = base + i * kStepBlock + threadIdx.x;
+            if (j < end) {
+                param[at(i)] = step_one<KIND>(sp, x[i], g[i], lr, m[i], v[i]);
+                store_state<KIND>(st, N, j, m[i], v[i]);
+            }
+        }
     }
 }
 
-// The same update with 16-byte accesses for the SH part (unpadded records,
-// L a multiple of 4, 16-byte aligned arrays): the step streams ~5 arrays of
-// L (1 + 3K) floats and is bound by HBM.
 template <int KIND>
-__global__ void k_step_vec(StepParams sp, float *sigma, float4 *sh4, const float *gs, const float4 *gsh4,
-                           float *state)
+void launch_step_kind(const StepParams &sp, int K, unsigned grid, float *sig, float *sh, const float *gs,
+                      const float *gsh, float *state, cudaStream_t s)
 {
-    const int64_t N = sp.L * (1 + sp.K3);
-    const int64_t n4 = sp.L * sp.K3 / 4;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < sp.L + n4;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        if (j < sp.L) {
-            float m = 0.f, v = 0.f;
-            load_state<KIND>(state, N, j, m, v);
-            sigma[j] = step_one<KIND>(sp, sigma[j], gs[j], sp.lr_sigma, m, v);
-            store_state<KIND>(state, N, j, m, v);
-        } else {
-            const int64_t u = j - sp.L;
-            float4 x = sh4[u];
-            const float4 g = gsh4[u];
-            float4 *m4 = nullptr, *v4 = nullptr;  // Adam m, v / RMSprop v (in m4)
-            if (KIND != POT_SGD) m4 = reinterpret_cast<float4 *>(state + sp.L) + u;
-            if (KIND == POT_ADAM) v4 = reinterpret_cast<float4 *>(state + N + sp.L) + u;
-            float4 m = make_float4(0.f, 0.f, 0.f, 0.f), v = m;
-            if (KIND == POT_RMSPROP) v = *m4;
-            if (KIND == POT_ADAM) {
-                m = *m4;
-                v = *v4;
-            }
-            x.x = step_one<KIND>(sp, x.x, g.x, sp.lr_sh, m.x, v.x);
-            x.y = step_one<KIND>(sp, x.y, g.y, sp.lr_sh, m.y, v.y);
-            x.z = step_one<KIND>(sp, x.z, g.z, sp.lr_sh, m.z, v.z);
-            x.w = step_one<KIND>(sp, x.w, g.w, sp.lr_sh, m.w, v.w);
-            sh4[u] = x;
-            if (KIND == POT_RMSPROP) *m4 = v;
-            if (KIND == POT_ADAM) {
-                *m4 = m;
-                *v4 = v;
-            }
-        }
+    switch (K) {
+    case 1: k_step<KIND, 1><<<grid, kStepBlock, 0, s>>>(sp, sig, sh, gs, gsh, state); break;
+    case 4: k_step<KIND, 4><<<grid, kStepBlock, 0, s>>>(sp, sig, sh, gs, gsh, state); break;
+    case 9: k_step<KIND, 9><<<grid, kStepBlock, 0, s>>>(sp, sig, sh, gs, gsh, state); break;
+    case 16: k_step<KIND, 16><<<grid, kStepBlock, 0, s>>>(sp, sig, sh, gs, gsh, state); break;
+    default: k_step<KIND, 25><<<grid, kStepBlock, 0, s>>>(sp, sig, sh, gs, gsh, state); break;
     }
 }
 
@@ -868,8 +863,6 @@ cudaError_t launch_step(pot_tree *t, int kind, float lr_sigma, float lr_sh, floa
 {
     StepParams sp;
     sp.L = t->n_leaves;
-    sp.K3 = 3 * t->K;
-    sp.stride = t->stride;
     sp.lr_sigma = lr_sigma;
     sp.lr_sh = lr_sh;
     sp.alpha = alpha;
@@ -879,26 +872,14 @@ cudaError_t launch_step(pot_tree *t, int kind, float lr_sigma, float lr_sh, floa
     sp.bc1 = (float)(1.0 - std::pow((double)beta1, (double)step));
     sp.bc2 = (float)(1.0 - std::pow((double)beta2, (double)step));
     if (sp.L == 0) return cudaSuccess;
-    const unsigned g = grid_n(sp.L * (1 + sp.K3));
+    int64_t units = (sp.L + kStepUnit - 1) / kStepUnit + (sp.L * 3 * t->K + kStepUnit - 1) / kStepUnit;
+    if (units > (1 << 30)) units = 1 << 30;
+    const unsigned g = (unsigned)units;
     float *sig = static_cast<float *>(t->sigma);
     float *sh = static_cast<float *>(t->sh);
-    const bool flat = sp.stride == sp.K3;
-    auto a16 = [](const void *q) { return ((uintptr_t)q & 15u) == 0; };
-    const bool vec = flat && sp.L % 4 == 0 && a16(sh) && a16(gsh) && (kind == POT_SGD || a16(state));
-    const unsigned gv = grid_n(sp.L + sp.L * sp.K3 / 4);
-#define POT_STEP(KIND)                                                                           \
-    if (vec) k_step_vec<KIND><<<gv, 256, 0, s>>>(sp, sig, reinterpret_cast<float4 *>(sh), gs,    \
-                                                  reinterpret_cast<const float4 *>(gsh), state); \
-    else if (flat) k_step<KIND, true><<<g, 256, 0, s>>>(sp, sig, sh, gs, gsh, state);            \
-    else k_step<KIND, false><<<g, 256, 0, s>>>(sp, sig, sh, gs, gsh, state);
-    if (kind == POT_SGD) {
-        POT_STEP(POT_SGD)
-    } else if (kind == POT_RMSPROP) {
-        POT_STEP(POT_RMSPROP)
-    } else {
-        POT_STEP(POT_ADAM)
-    }
-#undef POT_STEP
+    if (kind == POT_SGD) launch_step_kind<POT_SGD>(sp, t->K, g, sig, sh, gs, gsh, state, s);
+    else if (kind == POT_RMSPROP) launch_step_kind<POT_RMSPROP>(sp, t->K, g, sig, sh, gs, gsh, state, s);
+    else launch_step_kind<POT_ADAM>(sp, t->K, g, sig, sh, gs, gsh, state, s);
     count_launch();
     return cudaGetLastError();
 }
