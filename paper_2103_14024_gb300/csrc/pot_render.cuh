@@ -36,8 +36,8 @@ enum Lookup { kLookDense, kLookBrick, kLookAny };
 // pay for (256 x 256 f16 109 against 89 us, 800 x 800 f32 350 against 320 us)
 // and full launches do not notice (40 views: f16 5.68 against 5.65 ms, f32 7.31
 // against 7.32 ms).  72 registers (28 warps): 89 us, 340 us, 5.65 ms, 7.33 ms.
-// With bricks a step waits for two loads in turn, and 32 warps are better (one
-// full-HD view at depth 10: 768 against 801 us).
+// With bricks a step waits for two loads in turn, and more warps are better (one
+// full-HD view at depth 10: 28 warps 744, 32 warps 768, 24 warps 801 us).
 // Explicit rays need not have neighbours in their warp, and then every lane
 // brings its own lines: fewer resident warps keep more of them in L1.  4 blocks
 // against 6, 2^18 random pixels of 100 views on the depth-9 tree (one in four
@@ -50,7 +50,7 @@ constexpr int kBlock = 128;
 #ifndef POT_RENDER_MIN_BLOCKS
 #define POT_RENDER_MIN_BLOCKS 6
 #endif
-constexpr int render_min_blocks(Lookup l) { return l == kLookBrick ? 8 : POT_RENDER_MIN_BLOCKS; }
+constexpr int render_min_blocks(Lookup l) { return l == kLookBrick ? 7 : POT_RENDER_MIN_BLOCKS; }
 constexpr int rays_min_blocks(Lookup l) { return l == kLookAny ? 6 : 4; }  // explicit rays
 
 // Fixed-point ray times.  A walk measures time from the clip range's entry
