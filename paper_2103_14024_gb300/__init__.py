@@ -170,12 +170,21 @@ def _ptr(x):
     return C.c_void_p(x.data_ptr())
 
 
+_raw_stream = None  # (device) -> current stream handle, once CUDA is up
+
+
 def _stream(stream=None):
     if stream is None:
+        # a call's share of the host time: the raw handle of the current device's
+        # current stream, without a Stream object (3.9 -> 0.6 us)
+        global _raw_stream
         import torch
-        if torch.cuda.is_available():
-            return C.c_void_p(torch.cuda.current_stream().cuda_stream)
-        return None
+        if _raw_stream is None:
+            if not torch.cuda.is_available():
+                return None
+            torch.cuda.current_stream()  # initialises CUDA in torch
+            _raw_stream = torch._C._cuda_getCurrentRawStream
+        return C.c_void_p(_raw_stream(torch._C._cuda_getDevice()))
     if isinstance(stream, int):
         return C.c_void_p(stream)
     return C.c_void_p(stream.cuda_stream)
@@ -188,9 +197,7 @@ def _as_np(x, dtype):
 def make_cameras(cams_np) -> C.Array:
     """ctypes array of Camera from a numpy structured array with the synth.CAMERA_DTYPE layout."""
     cams_np = np.ascontiguousarray(cams_np)
-    arr = (Camera * len(cams_np))()
-    C.memmove(arr, cams_np.ctypes.data, 80 * len(cams_np))
-    return arr
+    return (Camera * len(cams_np)).from_buffer_copy(cams_np.view(np.uint8))
 
 
 def _opts(bg=(0.0, 0.0, 0.0), gamma=0.0, near=0.0, far=3.0e38, seg_count=None, leaf_touched=None,
