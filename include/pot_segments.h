@@ -39,7 +39,7 @@
  *             not fit in `capacity` (the forward's colours are still exact).
  * Sizing: about (mean leaf segments per ray) x n slots, plus one partly used
  * block of POT_SEGMENT_BLOCK slots per resident warp of the recording kernel
- * (3 blocks of 8 warps per SM: 3,648 warps on a 152-SM GB300); when the
+ * (at most 24 warps per SM: 3,648 warps on a 152-SM GB300); when the
  * records overflow, pot_render_backward_recorded detects it on the GPU and
  * computes the gradients by the walking backward instead (same result, no
  * host synchronisation).  A buffer holds one forward's records: reuse it only

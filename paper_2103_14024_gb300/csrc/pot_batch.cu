@@ -3,7 +3,7 @@
 //
 // The host groups the items by (SH coefficients, leaf dtype, layout of the cell
 // index); each group is one launch.  Every item contributes tiles of kTileW x kTileH pixels (as pot_render);
-// warps take tiles from one counter and find their item by binary search over
+// each warp renders the tile of its place in the grid and finds its item among
 // the items' first-tile offsets.  The per-ray code (walk + shading) is the
 // same as pot_render's, so a request renders bit-identically alone or in a mix.
 #include <algorithm>

@@ -1,11 +1,11 @@
 // pot_device.cuh -- device helpers of the PlenOctree render path (sm_103a).
 //
-// Geometry is fp32 throughout.  Plane-crossing times and plane-side tests use
-// error-free transformations (TwoSum, TwoProd via fma) so that a crossing time
-// is known to about 2^-46 relative and a segment length delta = t_exit - t to
-// about 2^-24 of delta itself.  Plain fp32 times would carry an absolute error
-// of about one ulp of t (~5e-7 at t ~ 4), which, multiplied by densities in the
-// thousands, would move a pixel by more than 1e-4.
+// Inputs are fp32.  A ray is set up with error-free transformations (TwoSum,
+// TwoProd via fma) and then walked in 64-bit integer times (Walker in
+// pot_render.cuh), so that a segment length delta = t_exit - t is known to about
+// 2^-24 of delta itself.  Plain fp32 times would carry an absolute error of about
+// one ulp of t (~5e-7 at t ~ 4), which, multiplied by densities in the thousands,
+// would move a pixel by more than 1e-4.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -108,12 +108,6 @@ __device__ __forceinline__ void two_prod(float a, float b, float &p, float &e)
 {
     p = __fmul_rn(a, b);
     e = __fmaf_rn(a, b, -p);
-}
-
-// (a - b) rounded once: hi parts cancel exactly when close.
-__device__ __forceinline__ float df_sub(df a, df b)
-{
-    return __fadd_rn(__fsub_rn(a.hi, b.hi), __fsub_rn(a.lo, b.lo));
 }
 
 // a < b, decided as (a.hi - b.hi) + (a.lo - b.lo) < 0 would be (the sign of a

@@ -1,8 +1,10 @@
 // pot_render.cuh -- forward render kernel of the PlenOctree path (sm_103a).
 //
 // One warp renders one tile of 32 rays at a time (4 x 8 pixels of a camera,
-// or 32 consecutive explicit rays); warps take tiles from a global counter
-// until none is left (persistent grid, one wave of resident blocks).  Per ray:
+// or 32 consecutive explicit rays).  Large calls: one wave of resident blocks,
+// whose warps take tiles from a global counter until none is left; calls whose
+// tiles are all resident at once: a tile per warp by its place in the grid, or
+// a part of one (next_tile).  Per ray:
 //   a1 pinhole ray (fp32 expression of the public header)
 //   a2 clip to the tree box and to [near, far]
 //   a3 locate the cell: one load from the tree's cell index (leaf, or the
@@ -10,9 +12,9 @@
 //      trees without one, a descent of the child array from the deepest
 //      ancestor the new voxel shares with the previous one (ancestor stack in
 //      shared memory)
-//   a4 exit time of the cell (double-float plane crossings, the earliest of
-//      three chosen with selects); an empty node of any size is crossed in one
-//      step (Sec. 3.2 "Rendering")
+//   a4 exit time of the cell (64-bit fixed point, the earliest of three upper
+//      faces); an empty node of any size is crossed in one step (Sec. 3.2
+//      "Rendering")
 //   a5 leaf fetch: sigma and the SH record in 32-byte (or 16-byte) vector loads
 //   a6 colour: sigmoid of the SH dot product, basis evaluated once per ray
 //      because it is constant along the ray (App. B.3.2)
