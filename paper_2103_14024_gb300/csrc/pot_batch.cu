@@ -41,6 +41,7 @@ struct BatchParams {
     int n_items;
     int64_t n_tiles;
     unsigned int *err;
+    int overlaps;  // launched while the previous group's last blocks run
 };
 
 template <int K, typename T, Lookup LOOKUP>
@@ -48,6 +49,8 @@ __global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) batch_kerne
 {
     POT_WALK_SHARED(K)
     const int lane = threadIdx.x & 31;
+    // the next group may start once this group's blocks have all started (see launch_batch_t)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // short blocks: every warp renders one tile and the block ends, so a
     // launch frees its SM slots tile by tile and launches of higher-priority
     // streams (small requests) start between them
@@ -110,8 +113,19 @@ __global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) batch_kerne
             if (it.t_final) it.t_final[px] = v.Tr;
         }
     }
+    // a group is not done before the groups ahead of it are
+    if (bp.overlaps && blockIdx.x == 0 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// Groups follow each other on the stream, and each ends with its longest rays
+// on a few SMs.  A group after the first is launched programmatically: its
+// blocks start as soon as all blocks of the previous group have (groups read
+// only descriptors and trees that were there before the first, and write
+// outputs of their own), and its block 0 waits for the previous group before it
+// ends, so that whatever follows the call on the stream waits for all groups.
+// Mixed requests on trees of degree 1, 2 and 3 (f16), one group each: 2 of
+// 256 x 256 88 -> 59 us, 3 of them 275 -> 168 us, 6 of up to 800 x 800 598 -> 517 us,
+// 24 of up to 1920 x 1080 3490 -> 3425 us.
 template <typename T>
 cudaError_t launch_batch_t(const BatchParams &bp, int K, Lookup look, bool need_stack, cudaStream_t s)
 {
@@ -124,9 +138,19 @@ cudaError_t launch_batch_t(const BatchParams &bp, int K, Lookup look, bool need_
     const int64_t blocks = (bp.n_tiles + kBlock / 32 - 1) / (kBlock / 32);
     if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
     const unsigned grid = (unsigned)(blocks > 0 ? blocks : 1);
-    fn<<<grid, kBlock, smem, s>>>(bp);
-    count_launch();
-    return cudaGetLastError();
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kBlock);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = bp.overlaps ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, bp);
+    if (e == cudaSuccess) count_launch();
+    return e;
 }
 
 }  // namespace
@@ -193,6 +217,7 @@ cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_
         bp.n_items = b - a;
         bp.n_tiles = last.tile_begin + (int64_t)last.tiles_x * ((last.H + kTileH - 1) / kTileH);
         bp.err = err;
+        bp.overlaps = g > 0;
         const pot_tree *t = items[order[a]].tree;
         const Lookup look = t->cell_kind == POT_CELLS_DENSE   ? kLookDense
                             : t->cell_kind == POT_CELLS_BRICK ? kLookBrick
