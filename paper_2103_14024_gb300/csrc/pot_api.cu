@@ -1073,7 +1073,6 @@ pot_status pot_render_mse_backward(const pot_tree *t, int64_t n, const float *or
     DeviceGuard g(t->device);
     cudaStream_t s = (cudaStream_t)stream;
     Tmp scratch;
-    POT_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), s), "memset loss");
     RenderParams p;
     fill_tree_params(p, t, opts);
     if (!p.err) return fail(POT_ERR_CUDA, "device error word unavailable");
@@ -1083,8 +1082,12 @@ pot_status pot_render_mse_backward(const pot_tree *t, int64_t n, const float *or
     p.near = near;
     p.far = far;
     p.n_tiles = (n + 31) / 32;
-    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles, &p.part_log2) ? 0 : 1, true, s), "scratch");
-    POT_CUDA(launch_mse_backward(p, target, rgb, loss, grad_sigma, grad_sh, t->desc.leaf_dtype, t->K, s),
+    // the loss's sum ahead of the tile counter, which a launch of one wave does without
+    static_assert(sizeof(LossSum) == 2 * sizeof(unsigned long long), "two zeroed counters hold the loss's sum");
+    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, 3, true, s), "scratch");
+    LossSum *sum = reinterpret_cast<LossSum *>(p.tile_counter);
+    p.tile_counter = one_wave(p.n_tiles, &p.part_log2) ? nullptr : p.tile_counter + 2;
+    POT_CUDA(launch_mse_backward(p, target, rgb, loss, sum, grad_sigma, grad_sh, t->desc.leaf_dtype, t->K, s),
              "mse backward");
     return POT_OK;
 }

@@ -154,9 +154,10 @@ struct BackwardParams {
     const float *rgb_fwd;  // NULL: computed by a first pass
     float *grad_sigma;
     float *grad_sh;
-    // fused MSE mode: dL/dC = mse_scale (C - target), L += sum (C - target)^2 mse_scale / 2
+    // fused MSE mode: dL/dC = mse_scale (C - target), L = sum (C - target)^2 / (3 n_rays)
     const float *target;
     float *loss;
+    LossSum *loss_sum;     // zero before the launch
     float *rgb_out;        // optional copy of C
     float mse_scale;
     // non-null: the kernel runs only if *run_if != 0 (the walking backward as
@@ -176,7 +177,12 @@ enum BackwardMode { kGradAndColour = 0, kGrad = 1, kMseTarget = 2 };
 
 // MODE kGradAndColour: dL/dC and C given; kGrad: dL/dC given, C from a first
 // walk; kMseTarget: C from a first walk, then dL/dC of the MSE against the
-// target, the loss summed per warp into *loss, C optionally written out.
+// target, C optionally written out.  The loss: each ray's squared error in float,
+// summed over a warp by shuffles, over the warp's tiles, the block and the grid in
+// double (one double reduction per block), and rounded once by the block that
+// finishes last.  A float sum of one rounded addition per warp was off by 1.1e-6 of
+// the loss at 20,011 rays (2,504 warps), by 2.6e-5 at 100,003 rays whose errors were
+// all alike.  The call of 20,011 rays 85.6 -> 87.4 us.
 template <int K, typename T, Lookup LOOKUP, int MODE>
 __global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kernel(const __grid_constant__ BackwardParams bp)
 {
@@ -187,6 +193,7 @@ __global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kern
     const T *sig_arr = static_cast<const T *>(p.sigma);
     const T *sh_arr = static_cast<const T *>(p.sh);
     int taken = 0, slot;
+    double wsum = 0.0;  // squared error of the warp's rays (MSE mode)
     for (unsigned long long tile; next_tile(p, lane, taken, tile, slot);) {
         const int64_t ray = (int64_t)tile * 32 + slot;
         float lsum = 0.f;  // this ray's squared error (MSE mode)
@@ -238,7 +245,22 @@ __global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kern
         if (MODE == kMseTarget) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-            if (lane == 0 && lsum != 0.f) atomicAdd(bp.loss, 0.5f * bp.mse_scale * lsum);
+            wsum += (double)lsum;
+        }
+    }
+    if (MODE == kMseTarget) {
+        __shared__ double part[kBlock / 32];
+        if (lane == 0) part[threadIdx.x >> 5] = wsum;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double sum = 0.0;
+            for (int w = 0; w < kBlock / 32; ++w) sum += part[w];
+            atomicAdd(&bp.loss_sum->sum, sum);
+            __threadfence();
+            if (atomicAdd(&bp.loss_sum->blocks, 1ull) == gridDim.x - 1) {  // every block's sum is in
+                __threadfence();
+                *bp.loss = (float)(*(volatile double *)&bp.loss_sum->sum / (3.0 * (double)p.n_rays));
+            }
         }
     }
 }
@@ -804,7 +826,7 @@ unsigned grid_n(int64_t n)
 cudaError_t launch_backward(const RenderParams &r, const float *grad_rgb, const float *rgb_fwd, float *grad_sigma,
                             float *grad_sh, int dtype, int K, cudaStream_t s)
 {
-    BackwardParams bp{r, grad_rgb, rgb_fwd, grad_sigma, grad_sh, nullptr, nullptr, nullptr, 0.f};
+    BackwardParams bp{r, grad_rgb, rgb_fwd, grad_sigma, grad_sh, nullptr, nullptr, nullptr, nullptr, 0.f};
     const int mode = rgb_fwd ? kGradAndColour : kGrad;
     switch (dtype) {
     case POT_F32: return launch_backward_t<float>(bp, K, mode, s);
@@ -813,10 +835,10 @@ cudaError_t launch_backward(const RenderParams &r, const float *grad_rgb, const 
     }
 }
 
-cudaError_t launch_mse_backward(const RenderParams &r, const float *target, float *rgb_out, float *loss,
+cudaError_t launch_mse_backward(const RenderParams &r, const float *target, float *rgb_out, float *loss, LossSum *sum,
                                 float *grad_sigma, float *grad_sh, int dtype, int K, cudaStream_t s)
 {
-    BackwardParams bp{r, nullptr, nullptr, grad_sigma, grad_sh, target, loss, rgb_out,
+    BackwardParams bp{r, nullptr, nullptr, grad_sigma, grad_sh, target, loss, sum, rgb_out,
                       2.f / (3.f * (float)r.n_rays)};
     switch (dtype) {
     case POT_F32: return launch_backward_t<float>(bp, K, kMseTarget, s);
@@ -850,7 +872,8 @@ cudaError_t launch_backward_recorded(const RenderParams &r, int64_t n_leaves, co
     }
     if (e != cudaSuccess) return e;
     // the fallback: every ray walked again, only if the records overflowed
-    BackwardParams bp{r, grad_rgb, rgb_fwd, grad_sigma, grad_sh, nullptr, nullptr, nullptr, 0.f, sb.state + 1};
+    BackwardParams bp{r, grad_rgb, rgb_fwd, grad_sigma, grad_sh, nullptr, nullptr, nullptr, nullptr, 0.f,
+                      sb.state + 1};
     switch (dtype) {
     case POT_F32: return launch_backward_t<float>(bp, K, kGradAndColour, s);
     case POT_F16: return launch_backward_t<__half>(bp, K, kGradAndColour, s);
