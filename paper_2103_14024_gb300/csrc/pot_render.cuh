@@ -229,7 +229,7 @@ struct Walker {
         float rh[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const bool neg = d[a] < 0.f;
+            const bool neg = move[a] && d[a] < 0.f;  // a still axis keeps its voxel, whatever its component's sign
             if (neg) flip |= 4u >> a;
             // the voxel entered: an fp32 estimate low by its error bound, so exact or too low (by one unless
             // the origin is far away), then exact tests of its upper plane's time (a point on a plane belongs
