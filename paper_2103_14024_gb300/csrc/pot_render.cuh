@@ -233,9 +233,12 @@ struct Walker {
             if (neg) flip |= 4u >> a;
             // the voxel entered: an fp32 estimate low by its error bound, so exact or too low (by one unless
             // the origin is far away), then exact tests of its upper plane's time (a point on a plane belongs
-            // to the voxel above)
+            // to the voxel above).  The bound: 8 roundings of 2^-24 (|t d| + |A|) / h (3 of tin.hi, for tin.lo;
+            // of A, the sum, 1 / h, the product and a subtraction one each), taken as 10, and on a mirrored
+            // axis 2 of R 2^-25 (R - g, less the margin), taken as 8
             const float g = __fmul_rn(__fmaf_rn(tin.hi, d[a], -Ahi[a]), invh);
-            const float margin = (fabsf(tin.hi * d[a]) + fabsf(Ahi[a])) * invh * 2.3841858e-7f + 1e-6f;
+            const float margin = (fabsf(tin.hi * d[a]) + fabsf(Ahi[a])) * invh * 5.9604645e-7f +
+                                 (1e-6f + (neg ? (float)R * 2.3841858e-7f : 0.f));
             int v = min(max(__float2int_rd((neg ? (float)R - g : g) - margin), 0), R - 1);
             hs[a] = fixed_time(fabsf(th[a]) * exp2_int(-p.depth), (neg ? -tl[a] : tl[a]) * exp2_int(-p.depth));
             if (!move[a]) {

@@ -1,4 +1,5 @@
-"""Where a walk starts: direction components too small to move a ray, against the float64 oracle."""
+"""Where a walk starts: direction components too small to move a ray, and origins just above a voxel's lower plane
+seen from the side that the ray leaves through, against the float64 oracle."""
 import itertools
 
 import numpy as np
@@ -46,3 +47,29 @@ def test_components_below_the_normal_floats(oracle_mod, small):
     o, d = np.array(o).astype(np.float32), np.array(d).astype(np.float32)
     assert (d != 0).all() and (d < 0).any()
     _compare(pot, oracle_mod, sc, o, d, ("none", "brick", "dense"))
+
+
+@pytest.mark.parametrize("depth", [5, 9, 12])
+@pytest.mark.parametrize("lo", [0.0, -0.25])
+def test_origins_just_above_low_planes(oracle_mod, depth, lo):
+    """Viewers inside the box, 1e-7 to 1e-3 voxels above a plane, looking down along one axis or more: the sliver of
+    the first voxel counts.  Densities make a voxel opaque, so that at depth 12 a skipped 1e-4 voxels would show."""
+    import paper_2103_14024_gb300 as pot
+    R = 1 << depth
+    h = 1.0 / R
+    rng = np.random.default_rng(depth)
+    v = rng.integers(1, max(2, R // 8), (400, 3))
+    v = np.unique(v, axis=0)
+    codes = np.sort(S.morton_encode(v[:, 0], v[:, 1], v[:, 2], depth))
+    sc = S.Scene(depth, (lo,) * 3, 1.0, 1, codes, np.full(len(codes), 30.0 * R, np.float32),
+                 rng.normal(0, 1, (len(codes), 4, 3)).astype(np.float32))
+    o, d = [], []
+    for i in range(4000):
+        c = v[i % len(v)]
+        f = np.where(rng.random(3) < 0.6, 10.0 ** rng.uniform(-7, -3, 3), rng.uniform(0.1, 0.9, 3))
+        o.append(lo + h * (c + f))
+        u = rng.normal(size=3)
+        down = rng.random(3) < 0.7
+        d.append(np.where(down, -np.abs(u), u))
+    o, d = np.array(o).astype(np.float32), np.array(d).astype(np.float32)
+    _compare(pot, oracle_mod, sc, o, d, ["none"] + ["brick"] * (3 <= depth <= 11) + ["dense"] * (depth <= 10))
