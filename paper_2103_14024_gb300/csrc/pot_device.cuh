@@ -114,21 +114,25 @@ __device__ __forceinline__ void two_prod(float a, float b, float &p, float &e)
 // rounded sum is the sign of the exact sum), with one addition fewer.
 __device__ __forceinline__ bool df_lt(df a, df b) { return __fsub_rn(a.hi, b.hi) < __fsub_rn(b.lo, a.lo); }
 
+// s / d for s = s0 + rest0, with rd = 1/d to a few ulp (the remainder is taken
+// exactly and corrected for).  hi and lo stay ordered where s0 cancels.
+__device__ __forceinline__ df quotient(float s0, float rest0, float d, float rd)
+{
+    const float s = __fadd_rn(s0, rest0), rest = __fadd_rn(__fsub_rn(s0, s), rest0);
+    float t = __fmul_rn(s, rd);
+    float r = __fadd_rn(__fmaf_rn(-t, d, s), rest);
+    return {t, __fmul_rn(r, rd)};
+}
+
 // Time t at which o + t d crosses plane k of one axis, i.e.
-// (lo + k h - o) / d, with A = lo - o given exactly as Ahi + Alo and rd = 1/d
-// to a few ulp (the remainder is taken exactly and corrected for).  hi and lo
-// stay ordered where the plane's offset from the origin cancels.
+// (lo + k h - o) / d, with A = lo - o given exactly as Ahi + Alo.
 __device__ __forceinline__ df cross_time(int k, float h, float Ahi, float Alo, float d, float rd)
 {
     float p, pe;
     two_prod((float)k, h, p, pe);
     float s0, e;
     two_sum(Ahi, p, s0, e);
-    const float rest0 = __fadd_rn(__fadd_rn(Alo, pe), e);
-    const float s = __fadd_rn(s0, rest0), rest = __fadd_rn(__fsub_rn(s0, s), rest0);
-    float t = __fmul_rn(s, rd);
-    float r = __fadd_rn(__fmaf_rn(-t, d, s), rest);
-    return {t, __fmul_rn(r, rd)};
+    return quotient(s0, __fadd_rn(__fadd_rn(Alo, pe), e), d, rd);
 }
 
 // Exact sign of (p - lo) - k h for fp32 p, lo, h and an integer k (|k| < 2^24):

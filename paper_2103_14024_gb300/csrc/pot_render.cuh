@@ -209,15 +209,14 @@ struct Walker {
             Ahi[a] *= p.frame.ws;
             Alo[a] *= p.frame.ws;
             rd[a] = move[a] ? rcp_ftz(d[a]) : 0.f;
-            // the box's two planes: A / d and A / d + size / d
-            df t0, t1;
-            t0.hi = __fmul_rn(Ahi[a], rd[a]);
-            t0.lo = __fmul_rn(__fadd_rn(__fmaf_rn(-t0.hi, d[a], Ahi[a]), Alo[a]), rd[a]);
+            // the box's two planes, A / d and (A + size) / d, the sum taken before the division: along a slow
+            // axis A / d and size / d are large, and their roundings would stay where they cancel
+            const df t0 = quotient(Ahi[a], Alo[a], d[a], rd[a]);
+            float s1, e1;
+            two_sum(Ahi[a], p.frame.size, s1, e1);
+            const df t1 = quotient(s1, __fadd_rn(Alo[a], e1), d[a], rd[a]);
             th[a] = __fmul_rn(p.frame.size, rd[a]);
             tl[a] = __fmul_rn(__fmaf_rn(-th[a], d[a], p.frame.size), rd[a]);
-            float e;
-            two_sum(t0.hi, th[a], t1.hi, e);
-            t1.lo = __fadd_rn(e, __fadd_rn(t0.lo, tl[a]));
             const bool neg = d[a] < 0.f;
             const df t_in = neg ? t1 : t0, t_out = neg ? t0 : t1;
             if (move[a] && df_lt(tin, t_in)) tin = t_in;

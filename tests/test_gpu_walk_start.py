@@ -1,5 +1,5 @@
-"""Where a walk starts: direction components too small to move a ray, and origins just above a voxel's lower plane
-seen from the side that the ray leaves through, against the float64 oracle."""
+"""Where a walk starts: direction components too small to move a ray, origins just above a voxel's lower plane seen
+from the side that the ray leaves through, and entries along slow axes, against the float64 oracle."""
 import itertools
 
 import numpy as np
@@ -71,5 +71,36 @@ def test_origins_just_above_low_planes(oracle_mod, depth, lo):
         u = rng.normal(size=3)
         down = rng.random(3) < 0.7
         d.append(np.where(down, -np.abs(u), u))
+    o, d = np.array(o).astype(np.float32), np.array(d).astype(np.float32)
+    _compare(pot, oracle_mod, sc, o, d, ["none"] + ["brick"] * (3 <= depth <= 11) + ["dense"] * (depth <= 10))
+
+
+@pytest.mark.parametrize("depth", [6, 9, 12])
+@pytest.mark.parametrize("slow", [1e-2, 1e-4, 1e-6])
+def test_entries_through_a_slow_axis(oracle_mod, depth, slow):
+    """Rays nearly parallel to two faces of the box that enter through one of them: the box's plane times on that axis
+    are large and nearly cancel.  A layer of opaque voxels under each face shows which voxel was entered."""
+    import paper_2103_14024_gb300 as pot
+    R = 1 << depth
+    h = 1.0 / R
+    rng = np.random.default_rng(int(-np.log10(slow)) + 100 * depth)
+    n = min(R, 64)
+    base = R // 2 - n // 2
+    i, j = np.meshgrid(np.arange(n) + base, np.arange(n) + base, indexing="ij")
+    v = np.unique(np.concatenate([np.roll(np.stack([np.full(i.size, layer), i.ravel(), j.ravel()], 1), a, axis=1)
+                                  for a in range(3) for layer in (0, R - 1)]), axis=0)
+    codes = np.sort(S.morton_encode(v[:, 0], v[:, 1], v[:, 2], depth))
+    sc = S.Scene(depth, (0.0,) * 3, 1.0, 1, codes, np.full(len(codes), 30.0 * R, np.float32),
+                 rng.normal(0, 1, (len(codes), 4, 3)).astype(np.float32))
+    o, d = [], []
+    for k in range(1500):
+        a, up = k % 3, k // 3 % 2
+        u = rng.normal(size=3)
+        u[(a + 1) % 3] = rng.choice([-1.0, 1.0])
+        u[a] = slow * rng.uniform(0.5, 2.0) * (1.0 if up else -1.0)
+        at = h * (base + n * rng.uniform(0.2, 0.8, 3))
+        at[a] = 0.0 if up else 1.0
+        o.append(at - u * rng.uniform(0.01, 1.0))
+        d.append(u)
     o, d = np.array(o).astype(np.float32), np.array(d).astype(np.float32)
     _compare(pot, oracle_mod, sc, o, d, ["none"] + ["brick"] * (3 <= depth <= 11) + ["dense"] * (depth <= 10))
