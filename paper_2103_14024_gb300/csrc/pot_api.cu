@@ -178,22 +178,22 @@ struct Tmp {
 
 // What a walk launch needs on the device besides its arrays: tile counters
 // (zeroed; none where one wave of warps takes all tiles) and the cameras (none
-// where they fit into the launch).  Both in one buffer and one copy.  In a
-// stream capture the cameras are copied from the caller's array by a node of
-// the graph: each replay reads the array as it is then, which neither launch
-// parameters nor this function's staging would.
+// where they fit into the launch), in one buffer.  The cameras are copied from
+// the caller's array itself: the runtime stages pageable memory before it returns,
+// a copy from pinned memory takes place in stream order, and a stream capture gets
+// a node that reads the array as it is at each replay, which launch parameters
+// would not.
 cudaError_t walk_scratch(RenderParams &p, Tmp &mem, const pot_camera *cams, int n_cams, int n_counters, bool few_ok,
                          cudaStream_t s)
 {
-    bool captured = false;
-    if (n_cams > 0) {
+    bool few = n_cams <= kFewCams && few_ok;
+    if (n_cams > 0 && few) {
         cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
         const cudaError_t e = cudaStreamIsCapturing(s, &st);
         if (e != cudaSuccess) return e;
-        captured = st != cudaStreamCaptureStatusNone;
+        few = st == cudaStreamCaptureStatusNone;
+        if (few) std::memcpy(p.few_cams, cams, sizeof(pot_camera) * n_cams);
     }
-    const bool few = n_cams <= kFewCams && few_ok && !captured;
-    if (n_cams > 0 && few) std::memcpy(p.few_cams, cams, sizeof(pot_camera) * n_cams);
     const size_t cam_bytes = few ? 0 : sizeof(pot_camera) * (size_t)n_cams;
     const size_t cnt_bytes = n_counters ? (sizeof(unsigned long long) * (size_t)n_counters + 255) / 256 * 256 : 0;
     if (cnt_bytes + cam_bytes == 0) return cudaSuccess;
@@ -202,12 +202,6 @@ cudaError_t walk_scratch(RenderParams &p, Tmp &mem, const pot_camera *cams, int 
     char *d = static_cast<char *>(mem.p);
     if (n_counters) p.tile_counter = reinterpret_cast<unsigned long long *>(d);
     if (cam_bytes) p.cams = reinterpret_cast<const pot_camera *>(d + cnt_bytes);
-    char h[20480];  // 200 cameras and their counters fit
-    if (!captured && cam_bytes && cnt_bytes + cam_bytes <= sizeof(h)) {
-        std::memset(h, 0, cnt_bytes);
-        std::memcpy(h + cnt_bytes, cams, cam_bytes);
-        return cudaMemcpyAsync(d, h, cnt_bytes + cam_bytes, cudaMemcpyHostToDevice, s);  // staged before it returns
-    }
     if (cnt_bytes) e = cudaMemsetAsync(d, 0, cnt_bytes, s);
     if (e == cudaSuccess && cam_bytes) e = cudaMemcpyAsync(d + cnt_bytes, cams, cam_bytes, cudaMemcpyHostToDevice, s);
     return e;
