@@ -121,6 +121,17 @@ bool is_device_ptr(const void *p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Whether p is plain host memory, which no copy of a stream writes to after the call that queued it has returned.
+bool is_pageable(const void *p)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return a.type == cudaMemoryTypeUnregistered;
+}
+
 }  // namespace
 
 // Stream-ordered scratch of the library comes from a memory pool per device
@@ -180,9 +191,9 @@ struct Tmp {
 // (zeroed; none where one wave of warps takes all tiles) and the cameras (none
 // where they fit into the launch), in one buffer.  The cameras are copied from
 // the caller's array itself: the runtime stages pageable memory before it returns,
-// a copy from pinned memory takes place in stream order, and a stream capture gets
-// a node that reads the array as it is at each replay, which launch parameters
-// would not.
+// a copy from pinned or managed memory takes place in stream order, and a stream
+// capture gets a node that reads the array as it is at each replay.  Launch
+// parameters, filled during the call, are for pageable memory outside a capture.
 cudaError_t walk_scratch(RenderParams &p, Tmp &mem, const pot_camera *cams, int n_cams, int n_counters, bool few_ok,
                          cudaStream_t s)
 {
@@ -191,7 +202,7 @@ cudaError_t walk_scratch(RenderParams &p, Tmp &mem, const pot_camera *cams, int 
         cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
         const cudaError_t e = cudaStreamIsCapturing(s, &st);
         if (e != cudaSuccess) return e;
-        few = st == cudaStreamCaptureStatusNone;
+        few = st == cudaStreamCaptureStatusNone && is_pageable(cams);
         if (few) std::memcpy(p.few_cams, cams, sizeof(pot_camera) * n_cams);
     }
     const size_t cam_bytes = few ? 0 : sizeof(pot_camera) * (size_t)n_cams;

@@ -34,7 +34,7 @@ def test_many_cameras(n_cams, size):
     pot.check()
 
 
-@pytest.mark.parametrize("n_cams", [9, 40, 257])
+@pytest.mark.parametrize("n_cams", [1, 8, 9, 40])
 def test_pinned_cameras_follow_the_stream(n_cams):
     import torch
     import paper_2103_14024_gb300 as pot
