@@ -7,6 +7,7 @@
 // the items' first-tile offsets.  The per-ray code (walk + shading) is the
 // same as pot_render's, so a request renders bit-identically alone or in a mix.
 #include <algorithm>
+#include <memory>
 #include <vector>
 
 #include "pot_render.cuh"
@@ -153,6 +154,25 @@ cudaError_t launch_batch_t(const BatchParams &bp, int K, Lookup look, bool need_
     return e;
 }
 
+// A captured copy reads its source at each replay, so the graph takes the descriptors over and frees them with
+// its last instance.  Outside a capture nothing changes hands.
+cudaError_t graph_takes(std::unique_ptr<std::vector<BatchItem>> &items, cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    cudaGraph_t graph = nullptr;
+    cudaError_t e = cudaStreamGetCaptureInfo(s, &st, nullptr, &graph, nullptr, nullptr, nullptr);
+    if (e != cudaSuccess || st != cudaStreamCaptureStatusActive) return e;
+    cudaUserObject_t obj = nullptr;
+    e = cudaUserObjectCreate(
+        &obj, items.get(), [](void *v) { delete static_cast<std::vector<BatchItem> *>(v); }, 1,
+        cudaUserObjectNoDestructorSync);
+    if (e != cudaSuccess) return e;
+    items.release();
+    e = cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove);
+    if (e != cudaSuccess) cudaUserObjectRelease(obj, 1);
+    return e;
+}
+
 }  // namespace
 
 // items: host array of n validated requests; groups by (K, dtype, cell index), stages the
@@ -166,7 +186,8 @@ cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_
         return (t->K * 4 + t->desc.leaf_dtype) * 4 + t->cell_kind;
     };
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return key(a) < key(b); });
-    std::vector<BatchItem> desc(n);
+    auto owned = std::make_unique<std::vector<BatchItem>>(n);
+    std::vector<BatchItem> &desc = *owned;
     std::vector<int> group_start;
     int64_t tiles = 0;
     for (int k = 0; k < n; ++k) {
@@ -204,7 +225,8 @@ cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_
     const int groups = (int)group_start.size() - 1;
     BatchItem *d_items = nullptr;
     cudaMemPool_t pool = nullptr;
-    cudaError_t e = scratch_pool(&pool);
+    cudaError_t e = graph_takes(owned, s);
+    if (e == cudaSuccess) e = scratch_pool(&pool);
     if (e == cudaSuccess)
         e = cudaMallocFromPoolAsync(reinterpret_cast<void **>(&d_items), sizeof(BatchItem) * (size_t)n, pool, s);
     if (e != cudaSuccess) return e;
