@@ -384,7 +384,10 @@ pot_status pot_tree_quantize(const pot_tree *tree, int32_t bits, pot_tree **out,
  * group's items.  Per-ray arithmetic
  * is pot_render's: a request's pixels are identical alone or in a batch.
  * items: host array; rgb [H][W][3] and t_final [H][W] (may be NULL) in device
- * memory; trees on the current device.                                    */
+ * memory; trees on the current device.  Groups run in ascending order of their
+ * keys; where items share output memory, what a later group writes stands, and
+ * within a group either item's may.  In a stream capture the graph keeps what it
+ * needs of items; trees and outputs have to outlive its replays.          */
 typedef struct pot_render_item {
     const pot_tree *tree;
     pot_camera cam;

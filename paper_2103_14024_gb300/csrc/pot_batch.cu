@@ -8,6 +8,7 @@
 // same as pot_render's, so a request renders bit-identically alone or in a mix.
 #include <algorithm>
 #include <memory>
+#include <utility>
 #include <vector>
 
 #include "pot_render.cuh"
@@ -122,7 +123,7 @@ __global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) batch_kerne
 // on a few SMs.  A group after the first is launched programmatically: its
 // blocks start as soon as all blocks of the previous group have (groups read
 // only descriptors and trees that were there before the first, and write
-// outputs of their own), and its block 0 waits for the previous group before it
+// outputs of their own, see outputs_overlap), and its block 0 waits for the previous group before it
 // ends, so that whatever follows the call on the stream waits for all groups.
 // Mixed requests on trees of degree 1, 2 and 3 (f16), one group each: 2 of
 // 256 x 256 88 -> 59 us, 3 of them 275 -> 168 us, 6 of up to 800 x 800 598 -> 517 us,
@@ -152,6 +153,25 @@ cudaError_t launch_batch_t(const BatchParams &bp, int K, Lookup look, bool need_
     const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, bp);
     if (e == cudaSuccess) count_launch();
     return e;
+}
+
+// Whether some outputs of the items overlap.  Then the groups do not: the order in which they write decides.
+bool outputs_overlap(const std::vector<BatchItem> &items)
+{
+    std::vector<std::pair<const float *, const float *>> r;
+    r.reserve(2 * items.size());
+    for (const BatchItem &b : items) {
+        const int64_t px = (int64_t)b.W * b.H;
+        r.emplace_back(b.rgb, b.rgb + 3 * px);
+        if (b.t_final) r.emplace_back(b.t_final, b.t_final + px);
+    }
+    std::sort(r.begin(), r.end());
+    const float *end = nullptr;
+    for (const auto &q : r) {
+        if (q.first < end) return true;
+        end = q.second;
+    }
+    return false;
 }
 
 // A captured copy reads its source at each replay, so the graph takes the descriptors over and frees them with
@@ -231,6 +251,7 @@ cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_
         e = cudaMallocFromPoolAsync(reinterpret_cast<void **>(&d_items), sizeof(BatchItem) * (size_t)n, pool, s);
     if (e != cudaSuccess) return e;
     e = cudaMemcpyAsync(d_items, desc.data(), sizeof(BatchItem) * n, cudaMemcpyHostToDevice, s);
+    const bool apart = groups > 1 && !outputs_overlap(desc);
     for (int g = 0; g < groups && e == cudaSuccess; ++g) {
         const int a = group_start[g], b = group_start[g + 1];
         const BatchItem &last = desc[b - 1];
@@ -239,7 +260,7 @@ cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_
         bp.n_items = b - a;
         bp.n_tiles = last.tile_begin + (int64_t)last.tiles_x * ((last.H + kTileH - 1) / kTileH);
         bp.err = err;
-        bp.overlaps = g > 0;
+        bp.overlaps = g > 0 && apart;
         const pot_tree *t = items[order[a]].tree;
         const Lookup look = t->cell_kind == POT_CELLS_DENSE   ? kLookDense
                             : t->cell_kind == POT_CELLS_BRICK ? kLookBrick
