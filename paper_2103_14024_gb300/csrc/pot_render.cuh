@@ -210,11 +210,14 @@ struct Walker {
             Alo[a] *= p.frame.ws;
             rd[a] = move[a] ? rcp_ftz(d[a]) : 0.f;
             // the box's two planes, A / d and (A + size) / d, the sum taken before the division: along a slow
-            // axis A / d and size / d are large, and their roundings would stay where they cancel
-            const df t0 = quotient(Ahi[a], Alo[a], d[a], rd[a]);
+            // axis A / d and size / d are large, and their roundings would stay where they cancel.  Planes out of
+            // reach have infinite times (their remainder, infinite too, would undo the comparisons)
+            df t0 = quotient(Ahi[a], Alo[a], d[a], rd[a]);
             float s1, e1;
             two_sum(Ahi[a], p.frame.size, s1, e1);
-            const df t1 = quotient(s1, __fadd_rn(Alo[a], e1), d[a], rd[a]);
+            df t1 = quotient(s1, __fadd_rn(Alo[a], e1), d[a], rd[a]);
+            if (fabsf(t0.hi) > 3.4e38f) t0.lo = 0.f;
+            if (fabsf(t1.hi) > 3.4e38f) t1.lo = 0.f;
             th[a] = __fmul_rn(p.frame.size, rd[a]);
             tl[a] = __fmul_rn(__fmaf_rn(-th[a], d[a], p.frame.size), rd[a]);
             const bool neg = d[a] < 0.f;

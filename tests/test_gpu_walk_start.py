@@ -104,3 +104,25 @@ def test_entries_through_a_slow_axis(oracle_mod, depth, slow):
         d.append(u)
     o, d = np.array(o).astype(np.float32), np.array(d).astype(np.float32)
     _compare(pot, oracle_mod, sc, o, d, ["none"] + ["brick"] * (3 <= depth <= 11) + ["dense"] * (depth <= 10))
+
+
+@pytest.mark.parametrize("small", [1.5e-38, 1e-37, 1e-36, 1e-32])
+def test_slow_axis_outside_its_slab(oracle_mod, small):
+    """An origin outside the box on an axis along which the ray hardly moves: the box's plane times leave the float
+    range, and the ray misses the box."""
+    import paper_2103_14024_gb300 as pot
+    lo, size = -1.0, 2.0
+    sc = S.scene_random(431, 5, 1, p_occ=0.35, lo=(lo,) * 3, size=size, sigma_mu=1.5)
+    rng = np.random.default_rng(6)
+    o, d = [], []
+    for k in range(600):
+        a = k % 3
+        u = rng.normal(size=3)
+        at = lo + size * rng.uniform(0.1, 0.9, 3)
+        start = at - 3.0 * u
+        start[a] = at[a] if k % 2 else rng.choice([-1, 1]) * 10.0 ** rng.uniform(0.1, 4.0)
+        u[a] = small * rng.choice([-1, 1])
+        o.append(start)
+        d.append(u)
+    o, d = np.array(o).astype(np.float32), np.array(d).astype(np.float32)
+    _compare(pot, oracle_mod, sc, o, d, ("none", "brick", "dense"))
