@@ -201,10 +201,12 @@ struct Walker {
             d[a] = dw[a] * ds;
             move[a] = fabsf(d[a]) >= 1.17549435e-38f;
             if (!move[a]) {
-                // -(lo - o) in [0, size), decided exactly
+                // -(lo - o) in [0, size), or in (0, size] heading down, decided exactly
                 const float s = -Ahi[a], e = -Alo[a];
-                const bool inside = (s > 0.f || (s == 0.f && e >= 0.f)) && (s < p.size || (s == p.size && e < 0.f));
-                if (!inside) return false;
+                const bool down = dw[a] < 0.f;
+                const bool above = s > 0.f || (s == 0.f && (e > 0.f || (e == 0.f && !down)));
+                const bool below = s < p.size || (s == p.size && (e < 0.f || (e == 0.f && down)));
+                if (!above || !below) return false;
             }
             Ahi[a] *= p.frame.ws;
             Alo[a] *= p.frame.ws;
@@ -244,7 +246,10 @@ struct Walker {
             int v = min(max(__float2int_rd((neg ? (float)R - g : g) - margin), 0), R - 1);
             hs[a] = fixed_time(fabsf(th[a]) * exp2_int(-p.depth), (neg ? -tl[a] : tl[a]) * exp2_int(-p.depth));
             if (!move[a]) {
-                v = min(max(voxel_exact(o[a], p.lo[a], h / p.frame.ws, invh * p.frame.ws, R), 0), R - 1);
+                const float wh = h / p.frame.ws;
+                v = min(max(voxel_exact(o[a], p.lo[a], wh, invh * p.frame.ws, R), 0), R - 1);
+                // a point on a plane belongs to the voxel that even the smallest component heads for
+                if (dw[a] < 0.f && v > 0 && sign_point_minus_plane(o[a], p.lo[a], v, wh) == 0) --v;
                 nx[a] = hs[a] = kTimeNever;
             } else {
                 for (;; ++v) {

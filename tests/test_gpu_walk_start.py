@@ -126,3 +126,23 @@ def test_slow_axis_outside_its_slab(oracle_mod, small):
         d.append(u)
     o, d = np.array(o).astype(np.float32), np.array(d).astype(np.float32)
     _compare(pot, oracle_mod, sc, o, d, ("none", "brick", "dense"))
+
+
+@pytest.mark.parametrize("small", [0.0, 1e-45, 1e-39, 1e-36])
+def test_side_of_a_plane(oracle_mod, small):
+    """An origin on a voxel's plane, or the box's, belongs to the side that even the smallest component heads for."""
+    import paper_2103_14024_gb300 as pot
+    lo, size = -1.0, 2.0
+    sc = S.scene_random(432, 5, 1, p_occ=0.35, lo=(lo,) * 3, size=size, sigma_mu=1.5)
+    rng = np.random.default_rng(7)
+    o, d = [], []
+    for k in range(990):
+        a = k % 3
+        u = rng.normal(size=3)
+        start = lo + size * rng.uniform(0.1, 0.9, 3) - 3.0 * u
+        start[a] = lo + size / 32 * (k // 6 % 33)
+        u[a] = small * (1.0 if k // 3 % 2 else -1.0)
+        o.append(start)
+        d.append(u)
+    o, d = np.array(o).astype(np.float32), np.array(d).astype(np.float32)
+    _compare(pot, oracle_mod, sc, o, d, ("none", "brick", "dense"))
