@@ -43,13 +43,14 @@ WalkFrame walk_frame(float size, int depth)
 {
     int e = 0;
     std::frexp(size, &e);  // size in [2^(e-1), 2^e)
-    const int k = std::min(1 - e, 126 - kTimeFrac);
+    const int k = std::min(1 - e, 126);
     WalkFrame f;
     f.ws = std::ldexp(1.f, k);
     f.size = size * f.ws;
     f.h = std::ldexp(f.size, -depth);
     f.invh = 1.f / f.h;
-    f.unit = std::ldexp(1.f, -k - kTimeFrac);
+    f.unit = std::ldexp(1.f, -k);
+    f.rate = 1.44269504089f * f.unit;
     return f;
 }
 

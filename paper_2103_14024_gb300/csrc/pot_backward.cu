@@ -86,13 +86,14 @@ struct GradVisitor {
     float ctot[3];    // C of the ray (background included)
     float prefix[3];  // sum over composited segments of w c
     float Tr;
+    float unit;       // the frame's
     float *grad_sigma;
     float *grad_sh;
     template <typename YT>
     __device__ __forceinline__ bool operator()(int leaf, float delta, const YT &Y)
     {
         float gx[3], gsd;
-        const bool pos = segment_terms<K, T>(sig_arr, sh_arr, leaf, delta, Y, g, ctot, prefix, Tr, gx, gsd);
+        const bool pos = segment_terms<K, T>(sig_arr, sh_arr, leaf, delta * unit, Y, g, ctot, prefix, Tr, gx, gsd);
         float *row = grad_sh + (int64_t)leaf * (3 * K);
 #if POT_BWD_AGG
         // lanes compositing the same leaf: sum over the group with a shuffle
@@ -204,6 +205,7 @@ __global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kern
         gv.sh_arr = sh_arr;
         gv.gamma = p.gamma;
         gv.Tr = 1.f;
+        gv.unit = p.frame.unit;
         gv.grad_sigma = bp.grad_sigma;
         gv.grad_sh = bp.grad_sh;
         if (has) {
@@ -221,7 +223,8 @@ __global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kern
                 for (int c = 0; c < 3; ++c) gv.ctot[c] = __ldg(bp.rgb_fwd + 3 * ray + c);
             }
         } else {
-            ShadeVisitor<K, T, false> sv{sig_arr, sh_arr, nullptr, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, nullptr};
+            ShadeVisitor<K, T, false> sv{sig_arr, sh_arr, nullptr, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, nullptr,
+                                         p.frame.rate};
             walk_rays<K, T, LOOKUP, false>(p, stk, ysm, wst, has, o, d, p.near, p.far, sv);
 #pragma unroll
             for (int c = 0; c < 3; ++c) gv.ctot[c] = fmaf(sv.Tr, p.bg[c], sv.col[c]);

@@ -106,7 +106,8 @@ __global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) batch_kerne
         }
         const T *sig_arr = static_cast<const T *>(it.sigma);
         const T *sh_arr = static_cast<const T *>(it.sh);
-        ShadeVisitor<K, T, false> v{sig_arr, sh_arr, nullptr, it.gamma, {0.f, 0.f, 0.f}, 1.f, 0, it.codebook};
+        ShadeVisitor<K, T, false> v{sig_arr, sh_arr, nullptr, it.gamma, {0.f, 0.f, 0.f}, 1.f, 0, it.codebook,
+                                    it.frame.rate};
         walk_rays<K, T, LOOKUP, true>(p, stk, ysm, wst, has, o, d, c->near, c->far, v);
         if (has) {
             const int64_t px = (int64_t)j * it.W + i;

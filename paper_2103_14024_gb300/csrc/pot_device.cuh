@@ -508,12 +508,13 @@ __device__ __forceinline__ void leaf_colour_dot(const T *sh, int64_t leaf, const
 // e^x = 2^(x log2 e) by the base-2 exponential unit, denormals flushed: a
 // transmittance or an exponential below 2^-126 counts as 0 here, and 1 / (1 + e)
 // stays exact to 2 ulp without the range checks that denormals would need.
-__device__ __forceinline__ float exp_ftz(float x)
+__device__ __forceinline__ float exp2_ftz(float x)
 {
     float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x * 1.44269504089f));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+__device__ __forceinline__ float exp_ftz(float x) { return exp2_ftz(x * 1.44269504089f); }
 
 // 1 / x to one ulp, denormals flushed.
 __device__ __forceinline__ float rcp_ftz(float x)

@@ -17,11 +17,12 @@ struct MaxWeightVisitor {
     float gamma;
     float Tr;
     float *max_w;
+    float rate;  // the frame's
     template <typename YT>
     __device__ __forceinline__ bool operator()(int leaf, float delta, const YT &)
     {
         const float sig = fmaxf(Store<T>::load_sigma(sig_arr, leaf), 0.f);
-        const float e = exp_ftz(-sig * delta);
+        const float e = exp2_ftz((-sig * delta) * rate);
         const float w = Tr * (1.f - e);
         atomicMax(reinterpret_cast<int *>(max_w + leaf), __float_as_int(fmaxf(w, 0.f)));
         Tr *= e;
@@ -40,7 +41,7 @@ __global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) visibility_
         float o[3], d[3], near, far;
         int64_t ray;
         const bool has = tile_ray<true>(p, tile, slot, o, d, near, far, ray);
-        MaxWeightVisitor<T> v{sig_arr, p.gamma, 1.f, max_w};
+        MaxWeightVisitor<T> v{sig_arr, p.gamma, 1.f, max_w, p.frame.rate};
         walk_rays<K, T, LOOKUP, true>(p, stk, ysm, wst, has, o, d, near, far, v);
     }
 }

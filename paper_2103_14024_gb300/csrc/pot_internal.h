@@ -62,13 +62,13 @@ inline FastDiv fast_div(uint32_t d)
 }
 
 // The tree's box in the scale of the walk: lengths times the power of two ws
-// that brings the box's edge into [1, 2) (exact products, whatever the box's
-// size; capped where a time unit's length would fall below the normal floats).
+// that brings the box's edge into [1, 2) (exact products, whatever the box's size).
 struct WalkFrame {
     float ws;       // scale
     float size, h;  // edges of the box and of a voxel, scaled
     float invh;     // 1 / h, scaled
-    float unit;     // world length of 2^-kTimeFrac scaled lengths
+    float unit;     // world length of a scaled length of 1
+    float rate;     // unit log2 e: a segment lets 2^-(rate sigma length) through, its length scaled
 };
 constexpr int kTimeFrac = 49;
 WalkFrame walk_frame(float size, int depth);

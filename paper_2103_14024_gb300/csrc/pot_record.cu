@@ -22,6 +22,7 @@ namespace {
 template <int K, typename T>
 struct RecordVisitor {
     ShadeVisitor<K, T, false> sv;
+    float unit;  // the frame's
     bool has;
     int leaf;
     float delta, T0, P0[3];
@@ -30,7 +31,7 @@ struct RecordVisitor {
     {
         has = true;
         leaf = l;
-        delta = dl;
+        delta = dl * unit;
         T0 = sv.Tr;
 #pragma unroll
         for (int c = 0; c < 3; ++c) P0[c] = sv.col[c];
@@ -58,7 +59,9 @@ __global__ void __launch_bounds__(kBlock, rays_min_blocks(LOOKUP))
         const int64_t ray = (int64_t)tile * 32 + part;
         const bool has = part < 32 && ray < p.n_rays;
         RecordVisitor<K, T> v;
-        v.sv = ShadeVisitor<K, T, false>{sig_arr, sh_arr, nullptr, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, nullptr};
+        v.sv = ShadeVisitor<K, T, false>{sig_arr, sh_arr, nullptr, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, nullptr,
+                                         p.frame.rate};
+        v.unit = p.frame.unit;
         v.has = false;
         Walker<K, T, LOOKUP> w;
         w.ysm = ysm;

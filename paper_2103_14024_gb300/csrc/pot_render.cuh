@@ -93,7 +93,9 @@ __device__ __forceinline__ float exp2_int(int x) { return __int_as_float((127 + 
 // One ray's walk through the octree (a2-a4) as resumable state: begin() sets
 // the ray up (clip, locate, first cell); cross_empty() and cross_leaf() advance
 // past the cell the ray is in, the latter calling vis(leaf, delta, Y) for a
-// segment of positive length (Y: the SH basis at the ray direction); all three
+// segment of positive length (delta in the frame's scale, a power of two from the
+// world's, which costs visitors that only need sigma delta nothing; Y: the SH basis
+// at the ray direction); all three
 // return false once the walk is over (vis returned true, far clip, or the ray
 // left the box).  The next cell is located before vis runs on the current one,
 // so that its load overlaps the shading.
@@ -129,7 +131,7 @@ struct Walker {
     int64_t t, tout;
     int q[3];              // mirrored voxel
     uint32_t flip;         // the mirror, in the form of the tree's cell lookup
-    float unit;            // world length of one time unit
+    float unit;            // scaled length of one time unit
     int cell;              // entry of voxel q: leaf >= 0, or an empty box (cell_code_*)
     int step_i;
     // rows of shared memory: the per-ray SH basis, and 1 / hs per axis (read
@@ -190,7 +192,7 @@ struct Walker {
         // the direction scaled to a length in [1, 2)
         const int el = (int)(__float_as_uint(len) >> 23) - 127;
         const float ds = exp2_int(-el), il = invlen * exp2_int(el);
-        unit = __fmul_rn(__fmul_rn(len, ds), p.frame.unit);
+        unit = __fmul_rn(len, ds) * (1.f / kTimeScale);
         float d[3], rd[3], Ahi[3], Alo[3], th[3], tl[3];  // A = lo - o exactly, 1 / d, time across the box
         bool move[3];
         // a2: clip range in scaled time (position o + t d)
@@ -219,7 +221,7 @@ struct Walker {
             two_sum(Ahi[a], p.frame.size, s1, e1);
             df t1 = quotient(s1, __fadd_rn(Alo[a], e1), d[a], rd[a]);
             if (fabsf(t0.hi) > 3.4e38f) t0.lo = 0.f;
-            if (fabsf(t1.hi) > 3.4e38f) t1.lo = 0.f;
+            if (!(fabsf(t1.hi) <= 3.4e38f)) t1 = {__fmul_rn(s1, rd[a]), 0.f};  // A may be infinite in a tiny box's scale
             th[a] = __fmul_rn(p.frame.size, rd[a]);
             tl[a] = __fmul_rn(__fmaf_rn(-th[a], d[a], p.frame.size), rd[a]);
             const bool neg = d[a] < 0.f;
@@ -493,13 +495,14 @@ struct ShadeVisitor {
     float Tr;
     int nseg;
     const void *cb;  // codebook (cb16 leaves only)
+    float rate;      // the frame's
     template <typename YT>
     __device__ __forceinline__ bool operator()(int leaf, float delta, const YT &Y)
     {
         const float sig = fmaxf(Store<T>::load_sigma(sig_arr, leaf), 0.f);
         float x[3];
         leaf_colour_dot<K, T>(sh_arr, leaf, Y, x, cb);
-        const float e = exp_ftz(-sig * delta);  // transmittance of the segment
+        const float e = exp2_ftz((-sig * delta) * rate);  // transmittance of the segment
         const float w = Tr * (1.f - e);
 #pragma unroll
         for (int c = 0; c < 3; ++c) col[c] = fmaf(w, sigmoidf_(x[c]), col[c]);
@@ -588,7 +591,8 @@ __global__ void __launch_bounds__(kBlock, CAMS ? render_min_blocks(LOOKUP) : ray
         float o[3], d[3], near, far;
         int64_t ray;
         const bool has = tile_ray<CAMS>(p, tile, slot, o, d, near, far, ray);
-        ShadeVisitor<K, T, COUNT> v{sig_arr, sh_arr, p.leaf_touched, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, p.codebook};
+        ShadeVisitor<K, T, COUNT> v{sig_arr, sh_arr, p.leaf_touched, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, p.codebook,
+                                    p.frame.rate};
         walk_rays<K, T, LOOKUP, CAMS>(p, stk, ysm, wst, has, o, d, near, far, v);
         if (has) store_ray<K, T, COUNT>(p, ray, v);
     }
