@@ -232,7 +232,9 @@ pot_status pot_sh_basis(int32_t K, int64_t n, const float *dirs, float *Y, pot_s
  *   T_i = exp(-sum_{j<i} max(sigma_j,0) delta_j),
  *   c_i = sigmoid(sum_k k_{i,k} Y_k(d)),
  * over the leaf segments of the ray clipped to the box and to [near, far];
- * stops after the first segment that leaves T < gamma.
+ * stops after the first segment that leaves T < gamma.  A segment that lets
+ * less than 2^-126 through lets nothing through; a NaN among a leaf's SH
+ * coefficients gives NaN in that channel of the rays that composite the leaf.
  *   cams [n_cams] in host memory, all with the same width and height;
  *   rgb [n_cams][H][W][3] float32 and t_final [n_cams][H][W] float32 (final
  *   transmittance T_N; may be NULL), host or device memory.               */
