@@ -54,7 +54,7 @@ WalkFrame walk_frame(float size, int depth)
     return f;
 }
 
-bool one_wave(int64_t n_tiles, int *part_log2)
+bool one_wave(int64_t n_tiles, int *part_log2, int resident_warps)
 {
     static std::atomic<int> sms[64];
     int dev = 0;
@@ -64,7 +64,7 @@ bool one_wave(int64_t n_tiles, int *part_log2)
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
         sms[dev].store(n, std::memory_order_relaxed);
     }
-    if (n_tiles > 16ll * n) return false;
+    if (n_tiles > (int64_t)resident_warps * n) return false;
     int l = 0;
     while (l < kMaxPartLog2 && (n_tiles << (l + 1)) <= (int64_t)kPartWarps * n) ++l;
     *part_log2 = l;
@@ -1050,7 +1050,8 @@ pot_status pot_render_backward(const pot_tree *t, int64_t n, const float *origin
     p.near = near;
     p.far = far;
     p.n_tiles = (n + 31) / 32;
-    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles, &p.part_log2) ? 0 : 1, true, s), "scratch");
+    const int n_counters = one_wave(p.n_tiles, &p.part_log2, kBackwardWarps) ? 0 : 1;
+    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, n_counters, true, s), "scratch");
     POT_CUDA(launch_backward(p, grad_rgb, rgb_fwd, grad_sigma, grad_sh, t->desc.leaf_dtype, t->K, s), "backward");
     return POT_OK;
 }
@@ -1092,7 +1093,7 @@ pot_status pot_render_mse_backward(const pot_tree *t, int64_t n, const float *or
     static_assert(sizeof(LossSum) == 2 * sizeof(unsigned long long), "two zeroed counters hold the loss's sum");
     POT_CUDA(walk_scratch(p, scratch, nullptr, 0, 3, true, s), "scratch");
     LossSum *sum = reinterpret_cast<LossSum *>(p.tile_counter);
-    p.tile_counter = one_wave(p.n_tiles, &p.part_log2) ? nullptr : p.tile_counter + 2;
+    p.tile_counter = one_wave(p.n_tiles, &p.part_log2, kBackwardWarps) ? nullptr : p.tile_counter + 2;
     POT_CUDA(launch_mse_backward(p, target, rgb, loss, sum, grad_sigma, grad_sh, t->desc.leaf_dtype, t->K, s),
              "mse backward");
     return POT_OK;
@@ -1188,7 +1189,8 @@ pot_status pot_render_backward_recorded(const pot_tree *t, int64_t n, const floa
     p.near = near;
     p.far = far;
     p.n_tiles = (n + 31) / 32;
-    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, one_wave(p.n_tiles, &p.part_log2) ? 0 : 1, true, s), "scratch");
+    const int n_counters = one_wave(p.n_tiles, &p.part_log2, kBackwardWarps) ? 0 : 1;
+    POT_CUDA(walk_scratch(p, scratch, nullptr, 0, n_counters, true, s), "scratch");
     const SegmentBuffer sb{static_cast<float4 *>(const_cast<void *>(records)), capacity,
                            reinterpret_cast<unsigned long long *>(const_cast<int64_t *>(seg_state))};
     // POT_SEGBWD_ORDER (read once): 1 (default) visits the records in leaf

@@ -172,18 +172,24 @@ cudaError_t compact_kept_leaves(const pot_tree *t, const float *score, float thr
 cudaError_t quantize_tree(const pot_tree *t, int bits, pot_tree *q, cudaStream_t s);
 cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_t s, unsigned int *err);
 
-// Whether n_tiles tiles are all resident at once in every walk kernel (16 warps
-// per SM at least): then the tiles go to the warps in order, and the launch needs
-// no tile counter, that is no allocation and no memset before it.  (With the
-// cameras in the launch too, one 256 x 256 view 88 -> 77 us, one 64 x 64 view
-// 26 -> 23 us.)  *part_log2: into how many warps a tile is split, as long as
+// Whether n_tiles tiles are all resident at once, resident_warps of them per SM:
+// then the tiles go to the warps in order, and the launch needs no tile counter,
+// that is no allocation and no memset before it.  (With the cameras in the launch
+// too, one 256 x 256 view 88 -> 77 us, one 64 x 64 view 26 -> 23 us.)  Forward
+// kernels hold 16 warps per SM at least; the backward kernels, whose registers are
+// cut for 12, would take two waves without a balance between them: 65,000 random
+// rays on the depth-8 degree-4 tree 345 -> 271 us, on the depth-9 degree-3 tree
+// 207 -> 195 us with the line at 12 instead of 16, 77,000 rays 347 -> 305 and
+// 209 -> 207 us.  *part_log2: into how many warps a tile is split, as long as
 // kPartWarps per SM are not filled (24: one 200 x 200 f32 view 235 -> 217 us, fused
 // training call of 20,011 rays 92 -> 84 us; 48: 201 and 109 us; 16: 235 and 86 us).
+// A split launch may take a second wave where a kernel holds fewer warps than that.
 #ifndef POT_PART_WARPS
 #define POT_PART_WARPS 24
 #endif
 constexpr int kPartWarps = POT_PART_WARPS, kMaxPartLog2 = 4;
-bool one_wave(int64_t n_tiles, int *part_log2);
+constexpr int kForwardWarps = 16, kBackwardWarps = 12;
+bool one_wave(int64_t n_tiles, int *part_log2, int resident_warps = kForwardWarps);
 
 // cameras interleaved per tile group in camera renders (POT_VIEW_GROUP overrides)
 int render_view_group(int n_cams);

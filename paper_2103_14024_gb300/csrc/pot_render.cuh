@@ -4,7 +4,7 @@
 // or 32 consecutive explicit rays).  Large calls: one wave of resident blocks,
 // whose warps take tiles from a global counter until none is left; calls whose
 // tiles are all resident at once: a tile per warp by its place in the grid, or
-// a part of one (next_tile).  Per ray:
+// a part of one (one_wave, next_tile).  Per ray:
 //   a1 pinhole ray (fp32 expression of the public header)
 //   a2 clip to the tree box and to [near, far]
 //   a3 locate the cell: one load from the tree's cell index (leaf, or the

@@ -1,6 +1,6 @@
 """Explicit-ray and filtering calls with more tiles than one wave of warps takes: warps draw tiles from a counter and
 reuse their rows, stack and record blocks.  Compared with the same rays in calls that are one wave each, at sizes
-around the line between the two (16 warps per SM, 32 rays each) and well above it, ragged."""
+around the lines between the two (16 warps per SM, 12 in the backward, 32 rays each) and well above them, ragged."""
 import pytest
 
 from paper_2103_14024_gb300 import synth as S
@@ -10,8 +10,8 @@ RAYS = dict(bg=(0.2, 0.4, 0.6), gamma=1e-3, near=0.2, far=8.0)
 PIECE = 30011
 
 
-def _wave(torch):
-    return 16 * torch.cuda.get_device_properties(0).multi_processor_count * 32
+def _wave(torch, warps):
+    return warps * torch.cuda.get_device_properties(0).multi_processor_count * 32
 
 
 def _close(torch, a, b):
@@ -20,11 +20,11 @@ def _close(torch, a, b):
 
 
 @pytest.mark.parametrize("cells", ["none", "brick", "dense"])
-@pytest.mark.parametrize("over", [0, 1, 31, 22179])
-def test_rays_above_one_wave(cells, over):
+@pytest.mark.parametrize("warps,over", [(12, 0), (12, 1), (16, 0), (16, 1), (16, 31), (16, 22179)])
+def test_rays_above_one_wave(cells, warps, over):
     import torch
     import paper_2103_14024_gb300 as pot
-    n = _wave(torch) + over
+    n = _wave(torch, warps) + over
     tree = pot.Tree.from_scene(S.scene_random(91, 5, 3, p_occ=0.35, sigma_mu=1.5, sigma_s=1.0, sh_std=0.8))
     tree.set_cell_index(cells)
     o, d = (torch.from_numpy(a).cuda() for a in S.random_rays(91, n, radius=3.0, spread=0.9))
