@@ -175,6 +175,16 @@ enum BackwardMode { kGradAndColour = 0, kGrad = 1, kMseTarget = 2 };
 // every ray meets a leaf (see rays_min_blocks); 5: 814 us; 6: 908 us
 #define POT_BACKWARD_MIN_BLOCKS 3
 #endif
+// With bricks or without an index a step waits for loads in turn, and where a
+// segment's own registers are few (K <= 4: 80 hold it without spills) 24 warps are
+// better, 10^6 random rays: depth 10, degree 1, no index 2564 -> 2280 us, bricks
+// 1631 -> 1501 us, degree 0 2409 -> 1940 and 1461 -> 1236 us, 2^18 rays about half
+// of that gain, up to 40,000 within 3 % (4 and 5 blocks: 2552, 2557 us).  At degree
+// 3, whose registers spill, 2^18 rays take 591 instead of 445 us.
+constexpr int backward_min_blocks(Lookup l, int K)
+{
+    return l == kLookAny && K <= 4 ? 6 : POT_BACKWARD_MIN_BLOCKS;
+}
 
 // MODE kGradAndColour: dL/dC and C given; kGrad: dL/dC given, C from a first
 // walk; kMseTarget: C from a first walk, then dL/dC of the MSE against the
@@ -185,7 +195,8 @@ enum BackwardMode { kGradAndColour = 0, kGrad = 1, kMseTarget = 2 };
 // the loss at 20,011 rays (2,504 warps), by 2.6e-5 at 100,003 rays whose errors were
 // all alike.  The call of 20,011 rays 85.6 -> 87.4 us.
 template <int K, typename T, Lookup LOOKUP, int MODE>
-__global__ void __launch_bounds__(kBlock, POT_BACKWARD_MIN_BLOCKS) backward_kernel(const __grid_constant__ BackwardParams bp)
+__global__ void __launch_bounds__(kBlock, backward_min_blocks(LOOKUP, K))
+    backward_kernel(const __grid_constant__ BackwardParams bp)
 {
     POT_WALK_SHARED(K)
     const RenderParams &p = bp.r;
