@@ -47,7 +47,7 @@ struct BatchParams {
 };
 
 template <int K, typename T, Lookup LOOKUP>
-__global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) batch_kernel(const BatchParams bp)
+__global__ void __launch_bounds__(kBlock, render_min_blocks<K, T>(LOOKUP)) batch_kernel(const BatchParams bp)
 {
     POT_WALK_SHARED(K)
     const int lane = threadIdx.x & 31;

@@ -31,7 +31,7 @@ struct MaxWeightVisitor {
 };
 
 template <int K, typename T, Lookup LOOKUP>
-__global__ void __launch_bounds__(kBlock, render_min_blocks(LOOKUP)) visibility_kernel(const __grid_constant__ RenderParams p, float *max_w)
+__global__ void __launch_bounds__(kBlock, render_min_blocks<K, T>(LOOKUP)) visibility_kernel(const __grid_constant__ RenderParams p, float *max_w)
 {
     POT_WALK_SHARED(K)
     const int lane = threadIdx.x & 31;

@@ -39,7 +39,11 @@ enum Lookup { kLookDense, kLookBrick, kLookAny };
 // and full launches do not notice (40 views: f16 5.68 against 5.65 ms, f32 7.31
 // against 7.32 ms).  72 registers (28 warps): 89 us, 340 us, 5.65 ms, 7.33 ms.
 // With bricks a step waits for two loads in turn, and more warps are better (one
-// full-HD view at depth 10: 28 warps 744, 32 warps 768, 24 warps 801 us).
+// full-HD view at depth 10: 28 warps 744, 32 warps 768, 24 warps 801 us), but float
+// records of degree 3 and 4 keep 24: at 72 registers their loads wait for one
+// another, or spill (nine 100 x 100 views of the depth-8 degree-4 tree 263 -> 221 us,
+// of the depth-9 degree-3 tree 360 -> 279 us, 20 of 800 x 800 2750 -> 2745 and
+// 3497 -> 3455 us; 16-bit records of degree 4 2230 -> 2249 us, so they stay at 28).
 // Explicit rays need not have neighbours in their warp, and then every lane
 // brings its own lines: fewer resident warps keep more of them in L1.  4 blocks
 // against 6, 2^18 random pixels of 100 views on the depth-9 tree (one in four
@@ -52,7 +56,11 @@ constexpr int kBlock = 128;
 #ifndef POT_RENDER_MIN_BLOCKS
 #define POT_RENDER_MIN_BLOCKS 6
 #endif
-constexpr int render_min_blocks(Lookup l) { return l == kLookBrick ? 7 : POT_RENDER_MIN_BLOCKS; }
+template <int K, typename T>
+constexpr int render_min_blocks(Lookup l)
+{
+    return l == kLookBrick && (K < 16 || sizeof(T) < 4) ? 7 : POT_RENDER_MIN_BLOCKS;
+}
 constexpr int rays_min_blocks(Lookup l) { return l == kLookAny ? 6 : 4; }  // explicit rays
 
 // Fixed-point ray times.  A walk measures time from the clip range's entry
@@ -579,7 +587,7 @@ __device__ __forceinline__ void store_ray(const RenderParams &p, int64_t ray, co
 // Forward render, one tile per warp at a time: the warp takes the next tile
 // once all 32 of its rays are done.
 template <int K, typename T, Lookup LOOKUP, bool CAMS, bool COUNT>
-__global__ void __launch_bounds__(kBlock, CAMS ? render_min_blocks(LOOKUP) : rays_min_blocks(LOOKUP))
+__global__ void __launch_bounds__(kBlock, CAMS ? render_min_blocks<K, T>(LOOKUP) : rays_min_blocks(LOOKUP))
     render_kernel(const __grid_constant__ RenderParams p)
 {
     POT_WALK_SHARED(K)
