@@ -1257,7 +1257,15 @@ pot_status pot_loss_mse(int64_t n, const float *rgb, const float *target, float 
     if (!is_device_ptr(loss) || (n > 0 && (!is_device_ptr(rgb) || !is_device_ptr(target))) ||
         (grad_rgb && !is_device_ptr(grad_rgb)))
         return fail(POT_ERR_INVALID_ARG, "pot_loss_mse takes device arrays only");
-    POT_CUDA(launch_mse(n, rgb, target, grad_rgb, loss, (cudaStream_t)stream), "loss");
+    cudaStream_t s = (cudaStream_t)stream;
+    if (n == 0) {
+        POT_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), s), "loss");
+        return POT_OK;
+    }
+    Tmp sum;
+    POT_CUDA(sum.alloc(sizeof(LossSum), s), "alloc scratch");
+    POT_CUDA(cudaMemsetAsync(sum.p, 0, sizeof(LossSum), s), "memset");
+    POT_CUDA(launch_mse(n, rgb, target, grad_rgb, loss, static_cast<LossSum *>(sum.p), s), "loss");
     return POT_OK;
 }
 

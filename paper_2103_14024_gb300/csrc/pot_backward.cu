@@ -149,6 +149,25 @@ struct GradVisitor {
     }
 };
 
+// The mean of a launch's squared errors: each warp's sum (in its first lane) joins its block's and the grid's in
+// double, and the block that adds the last one writes the rounded mean.  Every thread of every block calls it.
+template <int BLOCK>
+__device__ __forceinline__ void finish_loss(double warp_sum, LossSum *s, double count, float *loss)
+{
+    __shared__ double part[BLOCK / 32];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = warp_sum;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    double sum = 0.0;
+    for (int w = 0; w < BLOCK / 32; ++w) sum += part[w];
+    atomicAdd(&s->sum, sum);
+    __threadfence();
+    if (atomicAdd(&s->blocks, 1ull) == gridDim.x - 1) {  // every block's sum is in
+        __threadfence();
+        *loss = (float)(*(volatile double *)&s->sum / count);
+    }
+}
+
 struct BackwardParams {
     RenderParams r;
     const float *grad_rgb;
@@ -262,21 +281,7 @@ __global__ void __launch_bounds__(kBlock, backward_min_blocks(LOOKUP, K))
             wsum += (double)lsum;
         }
     }
-    if (MODE == kMseTarget) {
-        __shared__ double part[kBlock / 32];
-        if (lane == 0) part[threadIdx.x >> 5] = wsum;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double sum = 0.0;
-            for (int w = 0; w < kBlock / 32; ++w) sum += part[w];
-            atomicAdd(&bp.loss_sum->sum, sum);
-            __threadfence();
-            if (atomicAdd(&bp.loss_sum->blocks, 1ull) == gridDim.x - 1) {  // every block's sum is in
-                __threadfence();
-                *bp.loss = (float)(*(volatile double *)&bp.loss_sum->sum / (3.0 * (double)p.n_rays));
-            }
-        }
-    }
+    if (MODE == kMseTarget) finish_loss<kBlock>(wsum, bp.loss_sum, 3.0 * (double)p.n_rays, bp.loss);
 }
 
 template <typename T>
@@ -794,9 +799,11 @@ void launch_step_kind(const StepParams &sp, int K, unsigned grid, float *sig, fl
 }
 
 // ---- MSE loss of a ray batch: L = mean over n*3 of (rgb - target)^2 --------
-__global__ void k_mse(int64_t n3, const float *rgb, const float *target, float *grad, float *loss)
+// (the blocks' sums joined in double: float reductions of up to 4,096 blocks were off
+// by 8e-7 of the loss at 200,003 random rays and by 4.6e-5 at 2^20 whose errors were
+// all alike; a training step of 2^18 rays 1529 -> 1533 us)
+__global__ void k_mse(int64_t n3, const float *rgb, const float *target, float *grad, LossSum *sum, float *loss)
 {
-    __shared__ float part[kFlatBlock / 32];
     const float scale = 2.f / (float)n3;
     float acc = 0.f;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n3; j += (int64_t)gridDim.x * blockDim.x) {
@@ -806,13 +813,7 @@ __global__ void k_mse(int64_t n3, const float *rgb, const float *target, float *
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float s = 0.f;
-        for (int w = 0; w < kFlatBlock / 32; ++w) s += part[w];
-        atomicAdd(loss, s / (float)n3);
-    }
+    finish_loss<kFlatBlock>((double)acc, sum, (double)n3, loss);
 }
 
 // ---- pixel rays (the camera expression of the public header) ----------------
@@ -936,11 +937,10 @@ cudaError_t launch_step(pot_tree *t, int kind, float lr_sigma, float lr_sh, floa
     return cudaGetLastError();
 }
 
-cudaError_t launch_mse(int64_t n, const float *rgb, const float *target, float *grad, float *loss, cudaStream_t s)
+cudaError_t launch_mse(int64_t n, const float *rgb, const float *target, float *grad, float *loss, LossSum *sum,
+                       cudaStream_t s)
 {
-    cudaError_t e = cudaMemsetAsync(loss, 0, sizeof(float), s);
-    if (e != cudaSuccess || n == 0) return e;
-    k_mse<<<grid_n(3 * n), kFlatBlock, 0, s>>>(3 * n, rgb, target, grad, loss);
+    k_mse<<<grid_n(3 * n), kFlatBlock, 0, s>>>(3 * n, rgb, target, grad, sum, loss);
     count_launch();
     return cudaGetLastError();
 }

@@ -153,7 +153,7 @@ cudaError_t launch_sh_basis(int K, int64_t n, const float *dirs, float *Y, cudaS
 
 cudaError_t launch_backward(const RenderParams &r, const float *grad_rgb, const float *rgb_fwd, float *grad_sigma,
                             float *grad_sh, int dtype, int K, cudaStream_t s);
-// The squared error of a fused training call while its blocks add to it (16 bytes, zero before the launch).
+// The squared error of a batch while the blocks of a launch add to it (16 bytes, zero before the launch).
 struct LossSum {
     double sum;
     unsigned long long blocks;  // that have added theirs
@@ -162,7 +162,8 @@ cudaError_t launch_mse_backward(const RenderParams &r, const float *target, floa
                                 float *grad_sigma, float *grad_sh, int dtype, int K, cudaStream_t s);
 cudaError_t launch_step(pot_tree *t, int kind, float lr_sigma, float lr_sh, float alpha, float beta1, float beta2,
                         float eps, int step, const float *gs, const float *gsh, float *state, cudaStream_t s);
-cudaError_t launch_mse(int64_t n, const float *rgb, const float *target, float *grad, float *loss, cudaStream_t s);
+cudaError_t launch_mse(int64_t n, const float *rgb, const float *target, float *grad, float *loss, LossSum *sum,
+                       cudaStream_t s);
 cudaError_t launch_camera_rays(const pot_camera *d_cams, int n_cams, int W, int H, int64_t n, const int64_t *pixels,
                                float *o, float *d, unsigned *d_flag, cudaStream_t s);
 
