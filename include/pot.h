@@ -324,7 +324,8 @@ pot_status pot_camera_rays(const pot_camera *cams, int32_t n_cams, int64_t n, co
  * renderer and own all GPU memory -- a viewer on a fixed memory budget, a host
  * whose allocator hooks refuse allocations by libraries, a frame loop that
  * cannot pay for an allocator call -- cannot use pot_render, which allocates a
- * small scratch buffer (tile counter + device copy of the cameras) per call.
+ * small scratch buffer (tile counter, device copy of the cameras) in calls that
+ * are large, have more than 8 cameras or are captured.
  * This call takes that scratch from one fixed array inside the library
  * (256 B + 1024 camera records = 82,176 B per GPU, held until the process
  * exits) and makes no allocation at all.

@@ -45,13 +45,16 @@ enum Lookup { kLookDense, kLookBrick, kLookAny };
 // of the depth-9 degree-3 tree 360 -> 279 us, 20 of 800 x 800 2750 -> 2745 and
 // 3497 -> 3455 us; 16-bit records of degree 4 2230 -> 2249 us, so they stay at 28).
 // Explicit rays need not have neighbours in their warp, and then every lane
-// brings its own lines: fewer resident warps keep more of them in L1.  4 blocks
+// brings its own lines: with the dense index fewer resident warps keep more of them in L1.  4 blocks
 // against 6, 2^18 random pixels of 100 views on the depth-9 tree (one in four
 // meets a leaf): render_rays 368 against 400 us, where every ray meets a leaf
 // 725 against 934 us; the recording forward 440 against 494 and 860 against
 // 1118 us (3 and 2 blocks the same within 1 %, as their registers allow 4).
 // The descent of the child array, a chain of loads, wants 24 warps there (no
-// index, 2^18 random pixels: 736 against 805 us).
+// index, 2^18 random pixels: 736 against 805 us), and trees with bricks run the same
+// instance (depth 9, degree 3, 200,000 random rays with bricks / without an index:
+// 24 warps 350 / 497, 20 warps 374 / 545, 28 warps 334 / 487, 32 warps 425 / 559 us;
+// 50,000 rays 229 / 354, 222 / 340, 282 / 411, 362 / 501 us).
 constexpr int kBlock = 128;
 #ifndef POT_RENDER_MIN_BLOCKS
 #define POT_RENDER_MIN_BLOCKS 6
@@ -99,8 +102,8 @@ __device__ __forceinline__ int64_t fixed_time_since(df a, df tin)
 __device__ __forceinline__ float exp2_int(int x) { return __int_as_float((127 + x) << 23); }
 
 // One ray's walk through the octree (a2-a4) as resumable state: begin() sets
-// the ray up (clip, locate, first cell); cross_empty() and cross_leaf() advance
-// past the cell the ray is in, the latter calling vis(leaf, delta, Y) for a
+// the ray up (clip, locate, first cell); approach() and step() advance past the
+// cell the ray is in, an empty box or any, the latter calling vis(leaf, delta, Y) for a
 // segment of positive length (delta in the frame's scale, a power of two from the
 // world's, which costs visitors that only need sigma delta nothing; Y: the SH basis
 // at the ray direction); all three
