@@ -49,8 +49,10 @@ WalkFrame walk_frame(float size, int depth)
     f.size = size * f.ws;
     f.h = std::ldexp(f.size, -depth);
     f.invh = 1.f / f.h;
-    f.unit = std::ldexp(1.f, -k);
-    f.rate = 1.44269504089f * f.unit;
+    const int ku = std::min(k + kTimeFrac, kMaxUnitLog2);
+    f.unit = std::ldexp(1.f, -ku);
+    f.rest = std::ldexp(1.f, ku - k - kTimeFrac);
+    f.rate = 1.44269504089f * f.rest;
     return f;
 }
 

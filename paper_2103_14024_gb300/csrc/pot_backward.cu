@@ -86,14 +86,14 @@ struct GradVisitor {
     float ctot[3];    // C of the ray (background included)
     float prefix[3];  // sum over composited segments of w c
     float Tr;
-    float unit;       // the frame's
+    float rest;       // the frame's
     float *grad_sigma;
     float *grad_sh;
     template <typename YT>
     __device__ __forceinline__ bool operator()(int leaf, float delta, const YT &Y)
     {
         float gx[3], gsd;
-        const bool pos = segment_terms<K, T>(sig_arr, sh_arr, leaf, delta * unit, Y, g, ctot, prefix, Tr, gx, gsd);
+        const bool pos = segment_terms<K, T>(sig_arr, sh_arr, leaf, delta * rest, Y, g, ctot, prefix, Tr, gx, gsd);
         float *row = grad_sh + (int64_t)leaf * (3 * K);
 #if POT_BWD_AGG
         // lanes compositing the same leaf: sum over the group with a shuffle
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kBlock, backward_min_blocks(LOOKUP, K))
         gv.sh_arr = sh_arr;
         gv.gamma = p.gamma;
         gv.Tr = 1.f;
-        gv.unit = p.frame.unit;
+        gv.rest = p.frame.rest;
         gv.grad_sigma = bp.grad_sigma;
         gv.grad_sh = bp.grad_sh;
         if (has) {

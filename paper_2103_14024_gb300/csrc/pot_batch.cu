@@ -2,11 +2,12 @@
 // resolutions and outputs (the work list of a continuous-batching server).
 //
 // The host groups the items by (SH coefficients, leaf dtype, layout of the cell
-// index); each group is one launch.  Every item contributes tiles of kTileW x kTileH pixels (as pot_render);
+// index, rate of the walk's frame); each group is one launch.  Every item contributes tiles of kTileW x kTileH pixels (as pot_render);
 // each warp renders the tile of its place in the grid and finds its item among
 // the items' first-tile offsets.  The per-ray code (walk + shading) is the
 // same as pot_render's, so a request renders bit-identically alone or in a mix.
 #include <algorithm>
+#include <cmath>
 #include <memory>
 #include <utility>
 #include <vector>
@@ -44,6 +45,7 @@ struct BatchParams {
     int64_t n_tiles;
     unsigned int *err;
     int overlaps;  // launched while the previous group's last blocks run
+    float rate;    // the frames'
 };
 
 template <int K, typename T, Lookup LOOKUP>
@@ -107,7 +109,7 @@ __global__ void __launch_bounds__(kBlock, render_min_blocks<K, T>(LOOKUP)) batch
         const T *sig_arr = static_cast<const T *>(it.sigma);
         const T *sh_arr = static_cast<const T *>(it.sh);
         ShadeVisitor<K, T, false> v{sig_arr, sh_arr, nullptr, it.gamma, {0.f, 0.f, 0.f}, 1.f, 0, it.codebook,
-                                    it.frame.rate};
+                                    bp.rate};
         walk_rays<K, T, LOOKUP, true>(p, stk, ysm, wst, has, o, d, c->near, c->far, v);
         if (has) {
             const int64_t px = (int64_t)j * it.W + i;
@@ -204,7 +206,10 @@ cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_
     for (int i = 0; i < n; ++i) order[i] = i;
     auto key = [&](int i) {
         const pot_tree *t = items[i].tree;
-        return (t->K * 4 + t->desc.leaf_dtype) * 4 + t->cell_kind;
+        // the frames of a group share their rate (all but tiny boxes have the same): a register less per ray than
+        // one rate per item, 8 requests of 256 x 256 207 -> 183 us
+        const int tiny = -std::ilogb(walk_frame(t->desc.bbox_size, t->desc.depth).rest);
+        return ((t->K * 4 + t->desc.leaf_dtype) * 4 + t->cell_kind) * 64 + tiny;
     };
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return key(a) < key(b); });
     auto owned = std::make_unique<std::vector<BatchItem>>(n);
@@ -262,6 +267,7 @@ cudaError_t launch_render_batch(const pot_render_item *items, int n, cudaStream_
         bp.n_tiles = last.tile_begin + (int64_t)last.tiles_x * ((last.H + kTileH - 1) / kTileH);
         bp.err = err;
         bp.overlaps = g > 0 && apart;
+        bp.rate = last.frame.rate;
         const pot_tree *t = items[order[a]].tree;
         const Lookup look = t->cell_kind == POT_CELLS_DENSE   ? kLookDense
                             : t->cell_kind == POT_CELLS_BRICK ? kLookBrick

@@ -63,14 +63,18 @@ inline FastDiv fast_div(uint32_t d)
 
 // The tree's box in the scale of the walk: lengths times the power of two ws
 // that brings the box's edge into [1, 2) (exact products, whatever the box's size).
+// In a box below 2^-76 a time unit's world length would be below the normal
+// floats: there segment lengths stay larger by a power of two, 1 / rest, which
+// the constant of the transmittance takes back.
 struct WalkFrame {
     float ws;       // scale
     float size, h;  // edges of the box and of a voxel, scaled
     float invh;     // 1 / h, scaled
-    float unit;     // world length of a scaled length of 1
-    float rate;     // unit log2 e: a segment lets 2^-(rate sigma length) through, its length scaled
+    float unit;     // length of 2^-kTimeFrac scaled lengths
+    float rest;     // world length of a length of 1; 1 for all but tiny boxes
+    float rate;     // rest log2 e: a segment lets 2^-(rate sigma length) through
 };
-constexpr int kTimeFrac = 49;
+constexpr int kTimeFrac = 49, kMaxUnitLog2 = 126;
 WalkFrame walk_frame(float size, int depth);
 
 constexpr int kFewCams = 8;  // 640 bytes of launch parameters

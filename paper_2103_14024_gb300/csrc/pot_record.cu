@@ -22,7 +22,7 @@ namespace {
 template <int K, typename T>
 struct RecordVisitor {
     ShadeVisitor<K, T, false> sv;
-    float unit;  // the frame's
+    float rest;  // the frame's
     bool has;
     int leaf;
     float delta, T0, P0[3];
@@ -31,7 +31,7 @@ struct RecordVisitor {
     {
         has = true;
         leaf = l;
-        delta = dl * unit;
+        delta = dl * rest;
         T0 = sv.Tr;
 #pragma unroll
         for (int c = 0; c < 3; ++c) P0[c] = sv.col[c];
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kBlock, rays_min_blocks(LOOKUP))
         RecordVisitor<K, T> v;
         v.sv = ShadeVisitor<K, T, false>{sig_arr, sh_arr, nullptr, p.gamma, {0.f, 0.f, 0.f}, 1.f, 0, nullptr,
                                          p.frame.rate};
-        v.unit = p.frame.unit;
+        v.rest = p.frame.rest;
         v.has = false;
         Walker<K, T, LOOKUP> w;
         w.ysm = ysm;

@@ -104,9 +104,8 @@ __device__ __forceinline__ float exp2_int(int x) { return __int_as_float((127 + 
 // One ray's walk through the octree (a2-a4) as resumable state: begin() sets
 // the ray up (clip, locate, first cell); approach() and step() advance past the
 // cell the ray is in, an empty box or any, the latter calling vis(leaf, delta, Y) for a
-// segment of positive length (delta in the frame's scale, a power of two from the
-// world's, which costs visitors that only need sigma delta nothing; Y: the SH basis
-// at the ray direction); all three
+// segment of positive length (delta: times frame.rest the world's length; Y: the SH
+// basis at the ray direction); all three
 // return false once the walk is over (vis returned true, far clip, or the ray
 // left the box).  The next cell is located before vis runs on the current one,
 // so that its load overlaps the shading.
@@ -142,7 +141,7 @@ struct Walker {
     int64_t t, tout;
     int q[3];              // mirrored voxel
     uint32_t flip;         // the mirror, in the form of the tree's cell lookup
-    float unit;            // scaled length of one time unit
+    float unit;            // length of one time unit
     int cell;              // entry of voxel q: leaf >= 0, or an empty box (cell_code_*)
     int step_i;
     // rows of shared memory: the per-ray SH basis, and 1 / hs per axis (read
@@ -203,7 +202,7 @@ struct Walker {
         // the direction scaled to a length in [1, 2)
         const int el = (int)(__float_as_uint(len) >> 23) - 127;
         const float ds = exp2_int(-el), il = invlen * exp2_int(el);
-        unit = __fmul_rn(len, ds) * (1.f / kTimeScale);
+        unit = __fmul_rn(__fmul_rn(len, ds), p.frame.unit);
         float d[3], rd[3], Ahi[3], Alo[3], th[3], tl[3];  // A = lo - o exactly, 1 / d, time across the box
         bool move[3];
         // a2: clip range in scaled time (position o + t d)
@@ -506,7 +505,7 @@ struct ShadeVisitor {
     float Tr;
     int nseg;
     const void *cb;  // codebook (cb16 leaves only)
-    float rate;      // the frame's
+    float rate;      // the frame's, from the launch's parameters: an operand, not a register
     template <typename YT>
     __device__ __forceinline__ bool operator()(int leaf, float delta, const YT &Y)
     {
