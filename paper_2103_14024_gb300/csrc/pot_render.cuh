@@ -210,42 +210,40 @@ struct Walker {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             two_sum(p.lo[a], -o[a], Ahi[a], Alo[a]);
-            d[a] = dw[a] * ds;
-            move[a] = fabsf(d[a]) >= 1.17549435e-38f;
+            move[a] = dw[a] != 0.f;
             if (!move[a]) {
-                // -(lo - o) in [0, size), or in (0, size] heading down, decided exactly
+                // -(lo - o) in [0, size), decided exactly
                 const float s = -Ahi[a], e = -Alo[a];
-                const bool down = dw[a] < 0.f;
-                const bool above = s > 0.f || (s == 0.f && (e > 0.f || (e == 0.f && !down)));
-                const bool below = s < p.size || (s == p.size && (e < 0.f || (e == 0.f && down)));
-                if (!above || !below) return false;
+                const bool inside = (s > 0.f || (s == 0.f && e >= 0.f)) && (s < p.size || (s == p.size && e < 0.f));
+                if (!inside) return false;
             }
             Ahi[a] *= p.frame.ws;
             Alo[a] *= p.frame.ws;
-            rd[a] = move[a] ? rcp_ftz(d[a]) : 0.f;
+            // no component is so small that its times leave the float range: those below 2^-125 and 2^-126 |A| count
+            // as that much (their sign still decides the side of a plane that a ray starts on)
+            d[a] = copysignf(fmaxf(fabsf(dw[a] * ds), fmaf(fabsf(Ahi[a]), 1.1754944e-38f, 2.3509887e-38f)), dw[a]);
+            rd[a] = rcp_ftz(d[a]);
             // the box's two planes, A / d and (A + size) / d, the sum taken before the division: along a slow
-            // axis A / d and size / d are large, and their roundings would stay where they cancel.  Planes out of
-            // reach have infinite times (their remainder, infinite too, would undo the comparisons)
-            df t0 = quotient(Ahi[a], Alo[a], d[a], rd[a]);
+            // axis A / d and size / d are large, and their roundings would stay where they cancel
+            const df t0 = quotient(Ahi[a], Alo[a], d[a], rd[a]);
             float s1, e1;
             two_sum(Ahi[a], p.frame.size, s1, e1);
-            df t1 = quotient(s1, __fadd_rn(Alo[a], e1), d[a], rd[a]);
-            if (fabsf(t0.hi) > 3.4e38f) t0.lo = 0.f;
-            if (!(fabsf(t1.hi) <= 3.4e38f)) t1 = {__fmul_rn(s1, rd[a]), 0.f};  // A may be infinite in a tiny box's scale
+            const df t1 = quotient(s1, __fadd_rn(Alo[a], e1), d[a], rd[a]);
             th[a] = __fmul_rn(p.frame.size, rd[a]);
             tl[a] = __fmul_rn(__fmaf_rn(-th[a], d[a], p.frame.size), rd[a]);
-            const bool neg = d[a] < 0.f;
+            const bool neg = dw[a] < 0.f;
             const df t_in = neg ? t1 : t0, t_out = neg ? t0 : t1;
             if (move[a] && df_lt(tin, t_in)) tin = t_in;
             if (move[a] && df_lt(t_out, tend)) tend = t_out;
         }
-        if (!df_lt(tin, tend)) return false;
+        // (an offset beyond the floats: so far from a tiny box that no ray to it resolves it)
+        if (!df_lt(tin, tend) || !(fabsf(Ahi[0]) + fabsf(Ahi[1]) + fabsf(Ahi[2]) < 3.4e38f)) return false;
         tout = fixed_time_since(tend, tin);
         flip = 0;
         float rh[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const bool neg = move[a] && d[a] < 0.f;  // a still axis keeps its voxel, whatever its component's sign
+            const bool neg = dw[a] < 0.f;
             if (neg) flip |= 4u >> a;
             // the voxel entered: an fp32 estimate low by its error bound, so exact or too low (by one unless
             // the origin is far away), then exact tests of its upper plane's time (a point on a plane belongs
@@ -258,10 +256,7 @@ struct Walker {
             int v = min(max(__float2int_rd((neg ? (float)R - g : g) - margin), 0), R - 1);
             hs[a] = fixed_time(fabsf(th[a]) * exp2_int(-p.depth), (neg ? -tl[a] : tl[a]) * exp2_int(-p.depth));
             if (!move[a]) {
-                const float wh = h / p.frame.ws;
-                v = min(max(voxel_exact(o[a], p.lo[a], wh, invh * p.frame.ws, R), 0), R - 1);
-                // a point on a plane belongs to the voxel that even the smallest component heads for
-                if (dw[a] < 0.f && v > 0 && sign_point_minus_plane(o[a], p.lo[a], v, wh) == 0) --v;
+                v = min(max(voxel_exact(o[a], p.lo[a], h / p.frame.ws, invh * p.frame.ws, R), 0), R - 1);
                 nx[a] = hs[a] = kTimeNever;
             } else {
                 for (;; ++v) {
