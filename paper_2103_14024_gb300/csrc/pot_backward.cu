@@ -212,7 +212,7 @@ constexpr int backward_min_blocks(Lookup l, int K)
 // double (one double reduction per block), and rounded once by the block that
 // finishes last.  A float sum of one rounded addition per warp was off by 1.1e-6 of
 // the loss at 20,011 rays (2,504 warps), by 2.6e-5 at 100,003 rays whose errors were
-// all alike.  The call of 20,011 rays 85.6 -> 87.4 us.
+// all alike.  The call of 20,011 rays 85 -> 88 us.
 template <int K, typename T, Lookup LOOKUP, int MODE>
 __global__ void __launch_bounds__(kBlock, backward_min_blocks(LOOKUP, K))
     backward_kernel(const __grid_constant__ BackwardParams bp)
