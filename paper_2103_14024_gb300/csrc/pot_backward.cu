@@ -199,7 +199,7 @@ enum BackwardMode { kGradAndColour = 0, kGrad = 1, kMseTarget = 2 };
 // better, 10^6 random rays: depth 10, degree 1, no index 2564 -> 2280 us, bricks
 // 1631 -> 1501 us, degree 0 2409 -> 1940 and 1461 -> 1236 us, 2^18 rays about half
 // of that gain, up to 40,000 within 3 % (4 and 5 blocks: 2552, 2557 us).  At degree
-// 3, whose registers spill, 2^18 rays take 591 instead of 445 us.
+// 3, whose registers spill, 200,000 rays (depth 9, bricks) take 591 instead of 445 us.
 constexpr int backward_min_blocks(Lookup l, int K)
 {
     return l == kLookAny && K <= 4 ? 6 : POT_BACKWARD_MIN_BLOCKS;
